@@ -176,14 +176,25 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
     pb->bytes = precision == TSMM_PREC_BF16X3 ? (size_t)(pb->kp * pb->w * pb->ntiles) * 2 * 2
                                               : (size_t)(pb->kp * pb->w * pb->ntiles) * es;
     pb->data = nullptr;
+    pb->tc_data = nullptr;
+    pb->tc_min = nullptr;
     if (pb->bytes > 0) {
-        cudaError_t e = cudaMalloc(&pb->data, pb->bytes);
+        const bool tc = tc_pack(dtype, regime, precision, n, k);
+        const size_t off = (size_t)round_up((int64_t)pb->bytes, 256);
+        const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
+        cudaError_t e = cudaMalloc(&pb->data, tc ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float) : pb->bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             delete pb;
             return cuda_status(e);
         }
-        e = precision == TSMM_PREC_BF16X3
+        if (tc) {
+            pb->tc_data = static_cast<char *>(pb->data) + off;
+            pb->tc_min = reinterpret_cast<float *>(static_cast<char *>(pb->data) + off + pieces);
+        }
+        e = tc ? launch_pack_b_tc(k, n, static_cast<const float *>(B_dev), ldb, static_cast<float *>(pb->data), pb->kp,
+                                  (int)pb->w, pb->tc_data, pb->tc_min, static_cast<cudaStream_t>(stream))
+            : precision == TSMM_PREC_BF16X3
                 ? launch_pack_b_bf16x3(k, n, B_dev, ldb, pb->data, (int)pb->w, pb->kp / kX3KB,
                                        pb->ntiles, static_cast<cudaStream_t>(stream))
                 : launch_pack_b(dtype, k, n, B_dev, ldb, pb->data, pb->kp, pb->w, pb->ntiles,
@@ -341,7 +352,8 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         }
     } else if (regime == 1) {
         p->np = tall_np(n);
-        p->bm = tall_bm(dtype, p->np);
+        p->tc = tc_pack(dtype, regime, precision, n, k);
+        p->bm = p->tc ? kTcRows : tall_bm(dtype, p->np);
         p->kp = round_up(k, kTallBKS);
         p->slabs = (m + p->bm - 1) / p->bm;
         const int64_t kstages = p->kp / kTallBKS;
@@ -349,7 +361,7 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         const int64_t per_split = (int64_t)p->np * p->slabs * p->bm * (int64_t)es;
         int64_t max_splits = 65535;
         if (per_split > 0) max_splits = std::min<int64_t>(max_splits, max_workspace / per_split);
-        const int per_sm = tall_resident_blocks(dtype == TSMM_F64, p->np);
+        const int per_sm = p->tc ? 2 : tall_resident_blocks(dtype == TSMM_F64, p->np);
         int s = (kstages > 0 && p->slabs > 0)
                     ? choose_splits(p->slabs, kstages, sms, max_splits, per_sm)
                     : 1;
@@ -444,6 +456,9 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
     a.kchunk = p->kchunk;
     a.kp = p->kp;
     a.slabs = p->slabs;
+    a.np = p->np;
+    a.Bt = pb->tc_data;
+    a.bmin = pb->tc_min;
 
     const bool tma = aligned(A_dev, 16) && ((lda * (int64_t)es) % 16 == 0) && m < INT_MAX &&
                      k < INT_MAX && (lda * (int64_t)es) < (1LL << 40) && encoder() != nullptr;
@@ -563,6 +578,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }
+    if (p->tc) return cuda_status(launch_tall_tc(tma ? &p->tmap : nullptr, a, s));
     cudaError_t e = p->dtype == TSMM_F32 ? launch_tall_f32(tma, p->np, &p->tmap, a, s)
                                          : launch_tall_f64(tma, p->np, &p->tmap, a, s);
     return cuda_status(e);

@@ -71,6 +71,12 @@ cudaError_t launch_grouped_t(const GroupParams &gp, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// FP32 widths above 16 run on the tensor cores (launch_grouped_tc in tsmm_tall_tc.cu).
+template <typename T>
+constexpr bool grouped_width(int np) {
+    return sizeof(T) == 8 || np <= 16;
+}
+
 // Per-width dispatch of the grouped kernel: tensor-map A (tsmm_group_<dtype>.cu)
 // and, in its load form lv, an A that a tensor map cannot describe
 // (tsmm_group_async_<dtype>.cu), in translation units of their own.
@@ -78,7 +84,8 @@ template <typename T>
 cudaError_t launch_grouped_tma_dispatch(int np, const GroupParams &gp, cudaStream_t s) {
 #define TSMM_GROUP_CASE(NPV) \
     case NPV:                \
-        return launch_grouped_t<T, NPV, false, -1>(gp, s);
+        if constexpr (grouped_width<T>(NPV)) return launch_grouped_t<T, NPV, false, -1>(gp, s); \
+        return cudaErrorInvalidValue;
     switch (np) {
         TSMM_FOR_TALL_WIDTHS(TSMM_GROUP_CASE)
         default:
@@ -98,7 +105,8 @@ template <typename T>
 cudaError_t launch_grouped_async_dispatch(int np, int lv, const GroupParams &gp, cudaStream_t s) {
 #define TSMM_GROUP_CASE(NPV) \
     case NPV:                \
-        return launch_grouped_async_np<T, NPV>(lv, gp, s);
+        if constexpr (grouped_width<T>(NPV)) return launch_grouped_async_np<T, NPV>(lv, gp, s); \
+        return cudaErrorInvalidValue;
     switch (np) {
         TSMM_FOR_TALL_WIDTHS(TSMM_GROUP_CASE)
         default:

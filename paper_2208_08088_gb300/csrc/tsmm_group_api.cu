@@ -1,5 +1,5 @@
 // tsmm_execute_grouped: many pre-packed TSMMs in as few launches as possible.
-// Regime (i) problems are batched, per dtype, padded column count and kind of
+// Regime (i) problems are batched, per dtype, padded column count (MMA width on the tensor cores) and kind of
 // A (one a tensor map can describe, or one whose base or column stride is not
 // a multiple of 16 bytes, and then its load form), into launches of the
 // grouped kernel (up to
@@ -22,6 +22,7 @@
 namespace tsmm {
 cudaError_t launch_grouped_f32(int np, bool unaligned, int lv, const GroupParams &gp, cudaStream_t s);
 cudaError_t launch_grouped_f64(int np, bool unaligned, int lv, const GroupParams &gp, cudaStream_t s);
+cudaError_t launch_grouped_tc(int width, bool unaligned, const GroupParams &gp, cudaStream_t s);  // tsmm_tall_tc.cu
 }  // namespace tsmm
 
 using namespace tsmm;
@@ -91,12 +92,18 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
         if (!seen.insert(items[i].plan).second) return TSMM_ERR_INVALID_ARG;  // shared workspace
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // classes of groupable problems: (dtype, np, kind of A, load form) -> item indices
+    // classes of groupable problems: (dtype, np, kind of A, load form) -> item indices; for the tensor-core kernel
+    // (any A in one form) np is its MMA width and the load form kTcForm
+    constexpr int kTcForm = -2;
     std::map<std::tuple<int, int, int, int>, std::vector<int>> classes;
     for (int i = 0; i < count; ++i) {
         const int kind = group_kind(items[i]);
         if (kind != 0) {
             const tsmm_plan_t p = items[i].plan;
+            if (p->tc) {
+                classes[std::make_tuple((int)p->dtype, (int)tc_width(p->n), kind, kTcForm)].push_back(i);
+                continue;
+            }
             const int lv = kind == 2 ? async_load_variant(p->dtype == TSMM_F32, p->np, items[i].A_dev, items[i].lda)
                                      : -1;
             classes[std::make_tuple((int)p->dtype, p->np, kind, lv)].push_back(i);
@@ -157,12 +164,16 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
                 a.kchunk = p->kchunk;
                 a.kp = p->kp;
                 a.slabs = p->slabs;
+                a.np = p->np;
+                a.Bt = it.pb->tc_data;
+                a.bmin = it.pb->tc_min;
                 g.item_begin = total;
                 total += n_items;
             }
             gp->total_items = total;
-            cudaError_t e = dt == TSMM_F32 ? launch_grouped_f32(np, unaligned, lv, *gp, s)
-                                           : launch_grouped_f64(np, unaligned, lv, *gp, s);
+            cudaError_t e = lv == kTcForm    ? launch_grouped_tc(np, unaligned, *gp, s)
+                            : dt == TSMM_F32 ? launch_grouped_f32(np, unaligned, lv, *gp, s)
+                                             : launch_grouped_f64(np, unaligned, lv, *gp, s);
             if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TSMM_ERR_OUT_OF_MEMORY : TSMM_ERR_CUDA;
         }
     }

@@ -58,6 +58,17 @@ inline int tall_bm(tsmm_dtype d, int np) { return tall_block_rows(d == TSMM_F64,
 // tiles fit 136 registers), else 2 (the width 48's 8 x 12 tiles need ~160).
 constexpr int tall_resident_blocks(bool f64, int np) { return (!f64 && (np == 32 || np == 64)) ? 3 : 2; }
 
+// FP32 regime (i) with n > 16 runs on the tensor cores (tsmm_tall_tc.cuh): slabs of kTcRows rows, k in chunks of
+// kTcKB, MMA width n rounded up to 16.  The line lies at 16 because up to there the fma kernel streams A at the copy
+// rate (n = 16: 0.64 ms at m = k = 32768), above it does not (n = 20: 0.78 ms against 0.68); m and k need no line
+// (m = 2048, n = 32, k = 2048: 85 us against 25; m = 100000, n = 64, k = 64: 25 us both).
+constexpr int kTcRows = 128;
+constexpr int kTcKB = kTallBKS;
+inline int64_t tc_width(int64_t n) { return (n + 15) / 16 * 16; }
+inline bool tc_pack(tsmm_dtype d, int regime, int precision, int64_t n, int64_t k) {
+    return d == TSMM_F32 && regime == 1 && precision == 0 && n > 16 && k > 0;
+}
+
 // Load form of the regime (i) kernel for an A that a tensor map cannot describe
 // (its bulk/element-copy kernel): for FP32 widths of 16 and more with A's base
 // 16-byte aligned, lda mod 4 -- every column's offset within 16 bytes is then
@@ -105,6 +116,10 @@ struct tsmm_packed_b_s {
     int device;
     void *data;      // device storage, kp * w * ntiles elements
     size_t bytes;
+    // tensor-core form behind it in the same allocation (nullptr: none): per 32-row chunk of k three BF16 pieces of
+    // tc_width(n) columns, then one float per chunk, the smallest nonzero |B| in it
+    void *tc_data;
+    float *tc_min;
 };
 
 struct tsmm_plan_s {
@@ -121,6 +136,7 @@ struct tsmm_plan_s {
     int splits;      // k splits (S)
     int64_t kchunk;  // packed-B rows per split (multiple of kTallBKS)
     int64_t kp;      // padded k
+    bool tc;         // runs the tensor-core kernel
     // regime (ii)
     int64_t mtiles, ntiles;
     // device scratch owned by the plan
@@ -150,6 +166,9 @@ struct TallArgs {
     unsigned *status;
     int splits;
     int64_t kchunk, kp, slabs;
+    int np;             // row length of Bp, and of the workspace's partial tiles
+    const void *Bt;     // tensor-core form of B and its chunks' smallest nonzero magnitudes
+    const float *bmin;
 };
 
 // Launchers (return cudaSuccess or the launch error).  `tma` selects the
@@ -158,6 +177,9 @@ cudaError_t launch_tall_f32(bool tma, int np, const CUtensorMap *tmap, const Tal
                             cudaStream_t s);
 cudaError_t launch_tall_f64(bool tma, int np, const CUtensorMap *tmap, const TallArgs &a,
                             cudaStream_t s);
+
+// The tensor-core kernel; tmap == nullptr: an A that a tensor map cannot describe.
+cudaError_t launch_tall_tc(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s);
 
 struct RankArgs {
     int64_t m, n, k, lda, ldc, kp;
@@ -229,6 +251,9 @@ int choose_splits(int64_t slabs, int64_t kstages, int num_sms, int64_t max_split
 
 cudaError_t launch_pack_b(tsmm_dtype dt, int64_t k, int64_t n, const void *B, int64_t ldb,
                           void *dst, int64_t kp, int64_t w, int64_t ntiles, cudaStream_t s);
+// One launch writes the regime (i) panel and its tensor-core form.
+cudaError_t launch_pack_b_tc(int64_t k, int64_t n, const float *B, int64_t ldb, float *panel, int64_t kp, int np,
+                             void *tc_data, float *tc_min, cudaStream_t s);
 cudaError_t launch_scale(tsmm_dtype dt, int64_t m, int64_t n, double beta, void *C, int64_t ldc,
                          cudaStream_t s);
 cudaError_t launch_copy_columns(tsmm_dtype dt, const void *src, int64_t lds, int64_t m, int64_t k, void *dst,

@@ -2,6 +2,7 @@
 // row-major panels), and the alpha == 0 / k == 0 path C = beta * C0.
 #include "tsmm_device.cuh"
 #include "tsmm_internal.h"
+#include "tsmm_tc.cuh"
 
 namespace tsmm {
 
@@ -20,6 +21,43 @@ __global__ void pack_b_kernel(const T *__restrict__ B, int64_t k, int64_t n, int
         const int64_t j = t * w + (rem - p * w);
         dst[e] = (p < k && j < n) ? B[p + j * ldb] : T(0);
     }
+}
+
+// The regime (i) panel and its tensor-core form (tsmm_tall_tc.cuh) in one pass: block c takes the 32 rows of chunk c
+// (lanes along k, so B is read coalesced), writes the panel rows, the three BF16 pieces of every element at
+// (j/8)*512 + (kk/8)*128 + (j%8)*16 + (kk%8)*2 of its piece, and the chunk's smallest nonzero magnitude.
+__global__ void __launch_bounds__(256) pack_b_tc_kernel(const float *__restrict__ B, int64_t k, int64_t n, int64_t ldb,
+                                                        float *__restrict__ panel, int np, int w,
+                                                        unsigned char *__restrict__ pieces, float *__restrict__ cmin) {
+    __shared__ float t[kTcKB][kTallMaxN + 1];
+    __shared__ uint32_t smin;
+    const int64_t p0 = (int64_t)blockIdx.x * kTcKB;
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    if (threadIdx.x == 0) smin = 0xffffffffu;
+    __syncthreads();
+    uint32_t mn = 0xffffffffu;
+    for (int j = warp; j < kTallMaxN; j += 8) {
+        const float x = (p0 + lane < k && j < n) ? B[p0 + lane + (int64_t)j * ldb] : 0.f;
+        t[lane][j] = x;
+        mn = min(mn, __float_as_uint(x) * 2u - 1u);
+    }
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    if (lane == 0) atomicMin(&smin, mn);
+    __syncthreads();
+    for (int e = threadIdx.x; e < kTcKB * np; e += 256) panel[p0 * np + e] = t[e / np][e % np];
+    unsigned char *dst = pieces + (int64_t)blockIdx.x * (w * kTcKB * 6);
+    const int piece = w * kTcKB * 2;
+    for (int e = threadIdx.x; e < w * (kTcKB / 2); e += 256) {
+        const int j = e / (kTcKB / 2), kk = e % (kTcKB / 2) * 2;
+        uint32_t h, m, l;
+        split3_bf16x2(t[kk][j], t[kk + 1][j], h, m, l);
+        unsigned char *q = dst + (j / 8) * (kTcKB / 8 * 128) + (kk / 8) * 128 + (j % 8) * 16 + (kk % 8) * 2;
+        *reinterpret_cast<uint32_t *>(q) = h;
+        *reinterpret_cast<uint32_t *>(q + piece) = m;
+        *reinterpret_cast<uint32_t *>(q + 2 * piece) = l;
+    }
+    if (threadIdx.x == 0)
+        cmin[blockIdx.x] = smin == 0xffffffffu ? __uint_as_float(0x7f800000u) : __uint_as_float((smin + 1u) >> 1);
 }
 
 // C = beta * C0 (beta != 0) or C = 0 (beta == 0, C0 not read).
@@ -65,6 +103,14 @@ cudaError_t launch_pack_b(tsmm_dtype dt, int64_t k, int64_t n, const void *B, in
     else
         pack_b_kernel<double><<<grid_for(total, threads), threads, 0, s>>>(
             static_cast<const double *>(B), k, n, ldb, static_cast<double *>(dst), kp, w, total);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_b_tc(int64_t k, int64_t n, const float *B, int64_t ldb, float *panel, int64_t kp, int np,
+                             void *tc_data, float *tc_min, cudaStream_t s) {
+    if (kp == 0) return cudaSuccess;
+    pack_b_tc_kernel<<<(unsigned)(kp / kTcKB), 256, 0, s>>>(B, k, n, ldb, panel, np, (int)tc_width(n),
+                                                            static_cast<unsigned char *>(tc_data), tc_min);
     return cudaGetLastError();
 }
 

@@ -229,6 +229,10 @@ void tsmm_server_s::launch(double t) {
             const tsmm_plan_s &pl = reqs[i]->plan;
             const int64_t es = (int64_t)dtype_size(pl.dtype);
             const bool unaligned = reinterpret_cast<uintptr_t>(r.A_dev) % 16 != 0 || (r.lda * es) % 16 != 0;
+            if (pl.tc) {
+                by_class[8192 + (unaligned ? 128 : 0) + (int)tc_width(pl.n)].push_back(reqs[i]);
+                continue;
+            }
             const int form = unaligned ? 1 + (1 + async_load_variant(pl.dtype == TSMM_F32, pl.np, r.A_dev, r.lda)) : 0;
             by_class[pl.regime * 1024 + form * 128 + pl.np].push_back(reqs[i]);
         }

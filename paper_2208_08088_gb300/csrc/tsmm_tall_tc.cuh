@@ -1,0 +1,482 @@
+// Regime (i), FP32, n > 16, on the tensor cores at FP32 accuracy:
+// C[m x n] = alpha * A[m x k] * B[k x n] + beta * C0.
+//
+// The FMA pipes cannot stream A at HBM speed for these widths (n = 64 needs 215 TFLOP/s, the pipes have 80).
+// An FP32 value is the exact sum of three BF16 values (h + m + l, 8 significant bits each), so a product is the sum
+// of nine BF16 products, each exact in FP32; the six largest are accumulated on the tensor cores in FP32:
+//     l*h, h*l, m*m, m*h, h*m, then h*h
+// (the three left out are below 2^-25 of |a||b|, under the rounding of one FP32 fma).  A chunk of 32 k-columns starts
+// from a zero accumulator, smallest products first, so only the last two MMAs round at the size of the chunk's
+// sum; the chunk sums are then added in FP32 registers, rounded to nearest.  A chain of k fmas becomes a chain of
+// k/32 additions, and the error against exact products is smaller than the fma kernel's at every length.
+//
+// Measured, m = k = 32768, n = 64, calls back to back: 1.93 ms (fma kernel, 88 % of the FP32 pipe) -> 0.81 ms at 5.4
+// TB/s (0.70 ms, 6.1 TB/s, at the clock of a single call); n = 32: 0.98 -> 0.68 ms; n = 20: 0.78 -> 0.68 ms.  Relative
+// error (2-norm) against 64 bits 1.2e-6 -> 2.3e-7; k = 64: 1.4e-7 -> 6.3e-8.  Bound by HBM, then by power: the MMAs keep
+// the tensor pipe 40 % busy, the issue slots 50 %.  Two blocks of one item each per SM so that one block's start and
+// finish overlap the other's stream; four converter warps a block (eight spill at the registers left: 0.83 ms).  The MMA
+// warp stays converged and elects the issuing lane: a loop under `lane == 0` keeps every descriptor in vector registers
+// and took 100 cycles an MMA (0.80 -> 0.70 ms at n = 64).
+//
+// What the split cannot carry goes another way: a block whose item meets an infinity, a NaN, an overflow (seen as a
+// non-finite sum), or entries so small that a piece of a product could leave FP32's normal range (smallest
+// nonzero |a| times smallest nonzero |b| below 2^-100), recomputes its item with plain fmas (tall_tc_fallback)
+// before it stores anything, so results follow IEEE fma arithmetic there.
+//
+// Block: one work item = one slab of 128 rows x one k range (the split-K scheme of the fma kernel, same workspace,
+// counters and fixed summation order), 12 warps, two blocks per SM:
+//   warps 0-3   converters: thread = row; FP32 A from shared memory, split, pieces to tensor memory (tcgen05.st)
+//   warps 4-7   promoters: thread = row; chunk sums from tensor memory, added in registers; epilogue
+//   warp 8 (and 11: U)  producers of A: tensor copies, or (U) one bulk copy per column
+//   warp 9      tensor-memory owner and MMA issuer;  warp 10  producer of packed B chunks
+#pragma once
+#include "tsmm_internal.h"
+#include "tsmm_tc.cuh"
+
+namespace tsmm {
+
+
+template <int W, bool U>
+struct TallTcCfg {
+    static constexpr int BM = kTcRows;
+    static constexpr int KB = kTcKB;                          // k per chunk (one stage)
+    static constexpr int A_STRIDE = U ? BM + 8 : BM;          // floats per column slot
+    static constexpr int A_BYTES = KB * A_STRIDE * 4;
+    static constexpr int PIECE = W * KB * 2;                  // one BF16 piece of a chunk of B
+    static constexpr int B_BYTES = 3 * PIECE;
+    static constexpr int SBO = KB / 8 * 128;
+    static constexpr int BUDGET = 112 * 1024;                 // two blocks per SM
+    static constexpr int SB = 3;
+    static constexpr int SA_RAW = (BUDGET - SB * B_BYTES) / A_BYTES;
+    static constexpr int SA = SA_RAW > 6 ? 6 : SA_RAW;
+    static constexpr int OFF_B = SA * A_BYTES;
+    static constexpr int OFF_BAR = OFF_B + SB * B_BYTES;
+    static constexpr int NBAR = 2 * SA + 2 * SB + 6;
+    static constexpr int SMEM = OFF_BAR + NBAR * 8 + 32;
+    static constexpr int PRODUCERS = U ? 2 : 1;
+    static constexpr int THREADS = 384;
+    static constexpr int COL_A = 2 * W;                       // TMEM: 2 accumulators, then 2 x 3 pieces of 16 columns
+    static constexpr int TMEM_COLS = 256;
+    static_assert(SA >= 3, "A ring");
+    static_assert(COL_A + 96 <= TMEM_COLS, "tensor memory");
+    static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two blocks per SM");
+    static_assert(BM * (W / 2) * 4 <= SA * A_BYTES, "fallback exchange");
+};
+
+// Plain fma recomputation of columns [c0, c0 + HW) of one row of the item, from global memory (slow path).
+template <int HW>
+__device__ __forceinline__ void tall_tc_fallback(const TallArgs &a, int64_t row, int64_t k0, int64_t k1, int c0, float *out) {
+    float2 acc[HW / 2];
+#pragma unroll
+    for (int j = 0; j < HW / 2; ++j) acc[j] = make_float2(0.f, 0.f);
+    const bool in = row < a.m;
+    const float *Ap = static_cast<const float *>(a.A) + (in ? row : 0) + k0 * a.lda;
+    const float *Bp = static_cast<const float *>(a.Bp) + k0 * a.np + c0;
+    if (k1 > a.k) k1 = a.k;
+    for (int64_t p = k0; p < k1; ++p, Ap += a.lda, Bp += a.np) {
+        const float x = in ? __ldg(Ap) : 0.f;
+        const float2 x2 = make_float2(x, x);
+#pragma unroll
+        for (int j = 0; j < HW; j += 4) {
+            if (c0 + j < a.np) {
+                const float4 b = __ldg(reinterpret_cast<const float4 *>(Bp + j));
+                acc[j / 2] = __ffma2_rn(x2, make_float2(b.x, b.y), acc[j / 2]);
+                acc[j / 2 + 1] = __ffma2_rn(x2, make_float2(b.z, b.w), acc[j / 2 + 1]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < HW / 2; ++j) {
+        out[2 * j] = acc[j].x;
+        out[2 * j + 1] = acc[j].y;
+    }
+}
+
+template <int W, bool U>
+__device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const TallArgs &a, int64_t slab, int split) {
+    using Cfg = TallTcCfg<W, U>;
+    constexpr int SA = Cfg::SA, SB = Cfg::SB, KB = Cfg::KB, BM = Cfg::BM;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + Cfg::OFF_BAR);
+    uint64_t *afull = bar;             // [SA] FP32 A landed
+    uint64_t *aempty = afull + SA;     // [SA] converters have read it
+    uint64_t *bfull = aempty + SA;     // [SB] B chunk landed
+    uint64_t *bempty = bfull + SB;     // [SB] the MMAs have read it
+    uint64_t *conv = bempty + SB;      // [2] pieces of A in tensor memory
+    uint64_t *mdone = conv + 2;        // [2] the chunk's MMAs are complete
+    uint64_t *drained = mdone + 2;     // [2] accumulator read
+    unsigned *tslot = reinterpret_cast<unsigned *>(bar + Cfg::NBAR);
+    unsigned *flag = tslot + 1;
+    unsigned *abort_flag = tslot + 2;
+    unsigned *unsafe = tslot + 3;
+
+    const int warp = threadIdx.x / 32;
+    const int lane = threadIdx.x % 32;
+    const int64_t k0 = (int64_t)split * a.kchunk;
+    const int64_t k1 = (k0 + a.kchunk < a.kp) ? k0 + a.kchunk : a.kp;
+    const int iters = (int)((k1 - k0) / KB);
+    const int64_t i0 = slab * BM;
+
+    if (threadIdx.x == 0) {
+        if (!U) prefetch_tmap(tmA);
+        for (int s = 0; s < SA; ++s) {
+            mbar_init(&afull[s], Cfg::PRODUCERS);
+            mbar_init(&aempty[s], 4);
+        }
+        for (int s = 0; s < SB; ++s) {
+            mbar_init(&bfull[s], 1);
+            mbar_init(&bempty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&conv[b], 4);
+            mbar_init(&mdone[b], 1);
+            mbar_init(&drained[b], 4);
+        }
+        *abort_flag = 0u;
+        *unsafe = 0u;
+        fence_mbar_init();
+    }
+    if (warp == 9) tc_alloc(tslot, Cfg::TMEM_COLS);
+    tcf_before();
+    __syncthreads();
+    tcf_after();
+    const uint32_t tmem = *tslot;
+
+    if (warp >= 8) {
+        reg_dec<40>();
+        if (warp == 8 || (U && warp == 11)) {
+            // ------------------------------------------------ A
+            const uint64_t pol = policy_evict_first();
+            bool ok = true;
+            int it = 0;
+            if constexpr (!U) {
+                if (lane == 0) {
+                    for (; it < iters; ++it) {
+                        const int s = it % SA;
+                        if (it >= SA && !mbar_wait_bounded(&aempty[s], (uint32_t)((it / SA) & 1) ^ 1)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_arrive_expect_tx(&afull[s], Cfg::A_BYTES);
+                        tma_load_2d(smem + s * Cfg::A_BYTES, tmA, (int32_t)i0, (int32_t)(k0 + (int64_t)it * KB),
+                                    &afull[s], pol);
+                    }
+                }
+            } else {
+                // lane l < 16 of producer w moves column 16 w + l of each stage: one bulk copy of the aligned span
+                // around its rows (column_span_bytes); columns beyond k are zero-filled
+                const int rows = (int)((a.m - i0 < BM) ? a.m - i0 : BM);
+                const int abase = (int)((reinterpret_cast<uintptr_t>(a.A) / 4) & 3);
+                const int ldv = (int)((uint64_t)a.lda & 3);
+                const int q = (warp == 8 ? 0 : KB / 2) + lane;
+                for (; it < iters; ++it) {
+                    const int s = it % SA;
+                    if (it >= SA) {
+                        const bool got = mbar_wait_bounded(&aempty[s], (uint32_t)((it / SA) & 1) ^ 1);
+                        if (!__all_sync(0xffffffffu, got)) {
+                            ok = false;
+                            break;
+                        }
+                    }
+                    const int64_t p = k0 + (int64_t)it * KB + q;
+                    float *slot = reinterpret_cast<float *>(smem + s * Cfg::A_BYTES) + q * Cfg::A_STRIDE;
+                    const int d = (abase + (int)(p & 3) * ldv) & 3;
+                    const bool mine = lane < KB / 2;
+                    const uint32_t bytes = mine && p < a.k ? column_span_bytes<float>(rows, d) : 0u;
+                    if (mine && p >= a.k) {
+                        for (int r = 0; r < Cfg::A_STRIDE; r += 4)
+                            *reinterpret_cast<uint4 *>(slot + r) = make_uint4(0, 0, 0, 0);
+                        fence_proxy_async_smem();
+                    }
+                    const uint32_t sum = __reduce_add_sync(0xffffffffu, bytes);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_expect_tx(&afull[s], sum);
+                    __syncwarp();
+                    if (bytes != 0u)
+                        bulk_load(slot, static_cast<const float *>(a.A) + i0 + p * a.lda - d, bytes, &afull[s], pol);
+                }
+            }
+            if (!ok) {
+                if (lane == 0) atomicOr(a.status, kDevErrTimeout);
+                // copies in flight land before the block may exit
+                for (int q = it > SA ? it - SA : 0; q < it; ++q) mbar_wait_bounded(&afull[q % SA], (uint32_t)((q / SA) & 1));
+            }
+        } else if (warp == 10) {
+            // ------------------------------------------------ B
+            if (lane == 0) {
+                const uint64_t pol = policy_evict_last();
+                const unsigned char *Bt = static_cast<const unsigned char *>(a.Bt) + (k0 / KB) * Cfg::B_BYTES;
+                int it = 0;
+                bool ok = true;
+                for (; it < iters; ++it, Bt += Cfg::B_BYTES) {
+                    const int s = it % SB;
+                    if (it >= SB && !mbar_wait_bounded(&bempty[s], (uint32_t)((it / SB) & 1) ^ 1)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_arrive_expect_tx(&bfull[s], Cfg::B_BYTES);
+                    bulk_load(smem + Cfg::OFF_B + s * Cfg::B_BYTES, Bt, Cfg::B_BYTES, &bfull[s], pol);
+                }
+                if (!ok) {
+                    atomicOr(a.status, kDevErrTimeout);
+                    for (int q = it > SB ? it - SB : 0; q < it; ++q)
+                        mbar_wait_bounded(&bfull[q % SB], (uint32_t)((q / SB) & 1));
+                }
+            }
+        } else if (warp == 9) {
+            // ------------------------------------------------ MMAs
+            // the whole warp walks the loop (uniform operands), one elected lane issues
+            constexpr uint32_t idesc = tc_idesc_bf16(BM, W);
+            const uint64_t bdesc = tc_desc(smem_addr(smem + Cfg::OFF_B), Cfg::SBO);
+            bool ok = true;
+            int it = 0, s = 0;
+            uint32_t sph = 0;
+            for (; it < iters; ++it) {
+                const int b = it & 1;
+                const uint32_t par = (uint32_t)(it >> 1) & 1;
+                ok = mbar_wait_bounded(&bfull[s], sph) && mbar_wait_bounded(&conv[b], par) &&
+                     (it < 2 || mbar_wait_bounded(&drained[b], par ^ 1));
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tcf_after();
+                if (elect_one()) {
+                    const uint32_t d = tmem + b * W;
+                    const uint32_t at = tmem + Cfg::COL_A + b * 48;
+                    const uint64_t bd = bdesc + (uint64_t)(s * (Cfg::B_BYTES / 16));
+                    // (piece of A, piece of B), smallest products first
+                    constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+                    for (int q = 0; q < 6; ++q)
+#pragma unroll
+                        for (int ks = 0; ks < KB / 16; ++ks)
+                            tc_mma_ts(d, at + PA[q] * 16 + ks * 8, bd + (uint64_t)((PB[q] * Cfg::PIECE + ks * 256) / 16),
+                                      idesc, (q | ks) != 0);
+                    tc_commit(&bempty[s]);
+                    tc_commit(&mdone[b]);
+                }
+                __syncwarp();
+                if (++s == SB) {
+                    s = 0;
+                    sph ^= 1;
+                }
+            }
+            if (!ok && lane == 0) {
+                atomicOr(a.status, kDevErrTimeout);
+                atomicOr(abort_flag, 1u);
+            }
+            // nothing may still write tensor memory when it is freed (the last chunks' MMAs)
+            for (int q = it > 2 ? it - 2 : 0; q < it; ++q) mbar_wait_bounded(&mdone[q & 1], (uint32_t)(q >> 1) & 1);
+            __syncwarp();
+            tcf_before();
+            named_barrier(2, 160);  // with the promoters: every accumulator is read
+            tcf_after();
+            tc_dealloc(tmem, Cfg::TMEM_COLS);
+        }
+        return;
+    }
+
+    const int r = threadIdx.x % 128;
+    const int64_t row = i0 + r;
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    constexpr int HW = W / 2;
+    float *ex = reinterpret_cast<float *>(smem);  // fallback: the converters' half of the columns
+    const float alpha = static_cast<float>(a.alpha);
+    const float beta = static_cast<float>(a.beta);
+    const int n = (int)a.n;
+    const int64_t mpad = a.slabs * BM;
+    float *ws = static_cast<float *>(a.ws) + i0 + r;
+    // C = alpha*v + beta*C0 for G columns from c0 of this thread's row, the C0 loads issued ahead of the stores
+    auto store = [&](int c0, const float *v, auto g_tag) {
+        constexpr int G = decltype(g_tag)::value;
+        if (row >= a.m) return;
+        float *c = static_cast<float *>(a.C) + row + (int64_t)c0 * a.ldc;
+        float old[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) old[j] = (beta != 0.f && c0 + j < n) ? c[(int64_t)j * a.ldc] : 0.f;
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            if (c0 + j < n) {
+                float o = alpha * v[j];
+                if (beta != 0.f) o = fmaf(beta, old[j], o);
+                c[(int64_t)j * a.ldc] = o;
+            }
+    };
+    // split-K: the last arriver sums the S partials in the fixed order s = 0..S-1; all 256 threads take part, each one
+    // row and every other group of 8 columns, the loads of four splits in flight together
+    auto finish = [&](int half) {
+        named_barrier(1, 256);
+        if (threadIdx.x == 0) *flag = atomicAdd(a.tickets + slab, 1u) == (unsigned)(a.splits - 1) ? 1u : 0u;
+        named_barrier(1, 256);
+        if (*flag == 0u) return;
+        __threadfence();
+        for (int c0 = half * 8; c0 < n; c0 += 16) {
+            float sum[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum[j] = 0.f;
+            const float *src = ws + (int64_t)c0 * mpad;
+            for (int sp = 0; sp < a.splits; sp += 4) {
+                float t[4][8];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        t[q][j] =
+                            (sp + q < a.splits && c0 + j < n) ? ld_cg(src + ((int64_t)(sp + q) * a.np + j) * mpad) : 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (sp + q < a.splits) sum[j] += t[q][j];
+            }
+            store(c0, sum, std::integral_constant<int, 8>{});
+        }
+        if (threadIdx.x == 0) a.tickets[slab] = 0u;  // ready for the next launch on this stream
+    };
+    if (warp < 4) {
+        // ---------------------------------------------------- converters
+        reg_dec<72>();
+        float bmin = __uint_as_float(0x7f800000u);
+        {
+            const float *bm = a.bmin + k0 / KB;
+            for (int c = lane; c < iters; c += 32) bmin = fminf(bmin, __ldg(bm + c));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) bmin = fminf(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
+        }
+        // U: offsets within 16 bytes of the columns 0..3 mod 4 of a chunk
+        const int abase = (int)((reinterpret_cast<uintptr_t>(a.A) / 4) & 3);
+        const int ldv = (int)((uint64_t)a.lda & 3);
+        uint32_t amin = 0xffffffffu;  // smallest 2|x| - 1 over the nonzero x (bit patterns)
+        bool ok = true;
+        for (int it = 0; it < iters; ++it) {
+            const int s = it % SA, b = it & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&afull[s], (uint32_t)((it / SA) & 1)))) {
+                ok = false;
+                break;
+            }
+            const float *src = reinterpret_cast<const float *>(smem + s * Cfg::A_BYTES) + r;
+#pragma unroll
+            for (int h = 0; h < KB / 16; ++h) {
+                float x[16];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const int col = h * 16 + q;
+                    x[q] = U ? src[col * Cfg::A_STRIDE + ((abase + (q & 3) * ldv) & 3)] : src[col * BM];
+                }
+                uint32_t ph[8], pm[8], pl[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    amin = min(amin, __float_as_uint(x[2 * q]) * 2u - 1u);
+                    amin = min(amin, __float_as_uint(x[2 * q + 1]) * 2u - 1u);
+                    split3_bf16x2(x[2 * q], x[2 * q + 1], ph[q], pm[q], pl[q]);
+                }
+                if (h == 0) {
+                    // the pieces' place is free once the MMAs of two chunks ago are done
+                    if (it >= 2)
+                        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&mdone[b], ((uint32_t)(it >> 1) & 1) ^ 1));
+                    tcf_after();
+                } else {
+                    release_reads_to_async_copy();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&aempty[s]);
+                }
+                const uint32_t t = tlane + Cfg::COL_A + b * 48 + h * 8;
+                tc_st8(t, ph);
+                tc_st8(t + 16, pm);
+                tc_st8(t + 32, pl);
+            }
+            if (!ok) break;
+            tc_wait_st();
+            tcf_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&conv[b]);
+        }
+        if (!ok && lane == 0) {
+            atomicOr(a.status, kDevErrTimeout);
+            atomicOr(abort_flag, 1u);
+        }
+        const float amn = amin == 0xffffffffu ? __uint_as_float(0x7f800000u) : __uint_as_float((amin + 1u) >> 1);
+        constexpr float kTiny = 7.8886091e-31f;  // 2^-100
+        if (row < a.m && !(amn >= kTiny && bmin >= kTiny && amn * bmin >= kTiny)) *unsafe = 1u;
+        // every converter and promoter warp gets here (bounded waits); the flags are read between two barriers
+        named_barrier(1, 256);
+        const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
+        if (stop) return;  // tile not written; the host sees TSMM_ERR_TIMEOUT
+        if (redo) {
+            float part[HW];
+            tall_tc_fallback<HW>(a, row, k0, k1, 0, part);
+#pragma unroll
+            for (int j = 0; j < HW; ++j) ex[j * BM + r] = part[j];
+            named_barrier(1, 256);
+        }
+        if (a.splits > 1) finish(0);
+        return;
+    }
+
+    // -------------------------------------------------------- promoters
+        reg_inc<120>();
+        float acc[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) acc[j] = 0.f;
+        bool ok = true;
+        for (int it = 0; it < iters; ++it) {
+            const int b = it & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&mdone[b], (uint32_t)(it >> 1) & 1))) {
+                ok = false;
+                break;
+            }
+            tcf_after();
+#pragma unroll
+            for (int c = 0; c < W; c += 16) {
+                uint32_t v[16];
+                tc_ld16(tlane + b * W + c, v);
+                if (c + 16 == W) {
+                    tcf_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&drained[b]);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; j += 2) {
+                    const float2 t = __fadd2_rn(make_float2(acc[c + j], acc[c + j + 1]),
+                                                make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])));
+                    acc[c + j] = t.x;
+                    acc[c + j + 1] = t.y;
+                }
+            }
+        }
+        if (!ok && lane == 0) {
+            atomicOr(a.status, kDevErrTimeout);
+            atomicOr(abort_flag, 1u);
+        }
+        tcf_before();
+        named_barrier(2, 160);
+        float z = 0.f;  // 0 unless a sum is infinite or NaN
+#pragma unroll
+        for (int j = 0; j < W; ++j) z = fmaf(acc[j], 0.f, z);
+        if (row < a.m && z != 0.f) *unsafe = 1u;
+    named_barrier(1, 256);
+    const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
+    if (stop) return;
+    if (redo) {
+        tall_tc_fallback<HW>(a, row, k0, k1, HW, acc + HW);
+        named_barrier(1, 256);
+#pragma unroll
+        for (int j = 0; j < HW; ++j) acc[j] = ex[j * BM + r];
+    }
+    if (a.splits == 1) {
+#pragma unroll
+        for (int c = 0; c < W; c += 8) store(c, acc + c, std::integral_constant<int, 8>{});
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+        if (j < n) ws[((int64_t)split * a.np + j) * mpad] = acc[j];
+    __threadfence();
+    finish(1);
+}
+
+template <int W, bool U>
+__global__ void __launch_bounds__(TallTcCfg<W, U>::THREADS, 2) tall_tc_kernel(const __grid_constant__ CUtensorMap tmA, const TallArgs a) {
+    tall_tc_block<W, U>(&tmA, a, blockIdx.x, (int)blockIdx.y);
+}
+
+}  // namespace tsmm
