@@ -40,12 +40,14 @@
  *     aborts or throws; every failure is a status code.
  *   - Accuracy: every entry satisfies |C - C_exact| <= 4*k*u*(|alpha| sum_p
  *     |A[i,p]||B[p,j]| + |beta||C0[i,j]|) with u = 2^-24 (F32) / 2^-53 (F64).
- *     Products are accumulated with IEEE fma in the working precision, or, for
- *     F32 with 16 < n <= 64, on the tensor cores from exact splits of every
- *     entry into three BF16 values with all products down to 2^-25 of |a||b|
- *     (errors measured smaller than the fma chain's); inputs such a split cannot
- *     carry (infinities, NaNs, overflow, products below 2^-100) are computed
- *     with fma.  No TF32, no product of rounded inputs.
+ *     Products are accumulated with IEEE fma in the working precision, or on the
+ *     tensor cores from splits of every entry (errors measured smaller than the
+ *     fma chain's): F32 with 16 < n <= 64 from exact splits into three BF16
+ *     values with all products down to 2^-25 of |a||b|; F64 with 1 < n <= 64 and
+ *     256 <= k <= 2^20 from 56-bit fixed point cut into seven 8-bit digits whose
+ *     products are summed exactly.  Inputs such a split cannot carry within the
+ *     bound (infinities, NaNs, overflow, extreme or very unevenly scaled
+ *     entries) are found by the kernel and computed with fma.
  */
 #ifndef TSMM_H
 #define TSMM_H
@@ -123,9 +125,9 @@ TSMM_API const char *tsmm_last_cuda_error(void);
  * Packed layout (private to the library, described for test readers): the
  * n columns are cut into `ntiles` tiles of `w` columns (regime (i): one tile,
  * w = the kernel's padded column count, n rounded up to one of 1, 2, 4, 8, 16,
- * 24, 32, 48, 64; regime (ii): w = 64; for F32 with 16 < n <= 64 the handle
- * also holds, behind this storage and not counted in its size, the BF16 pieces
- * the tensor-core kernel reads).  Tile t is a
+ * 24, 32, 48, 64; regime (ii): w = 64; where the tensor cores serve
+ * the shape the handle also holds, behind this storage and not counted in its
+ * size, the pieces or digits of B that their kernel reads).  Tile t is a
  * row-major kp x w block (kp = k rounded up to the kernel's k granule) at
  * element offset t*kp*w; element (p, jj) of tile t holds B[p, t*w + jj], and is
  * +0.0 where p >= k or t*w + jj >= n.

@@ -92,9 +92,8 @@ namespace tsmm {
 // `overhead` is the per-block fixed cost (pipeline fill, reduction, epilogue)
 // in stage units.  Smallest S wins ties, which also keeps the workspace small.
 int choose_splits(int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits,
-                  int per_sm) {
+                  int per_sm, int64_t overhead) {
     const int64_t resident = (int64_t)per_sm * num_sms;
-    const int64_t overhead = 4;
     int64_t best_s = 1;
     double best_t = -1.0;
     const int64_t s_max = std::max<int64_t>(1, std::min<int64_t>(kstages, max_splits));
@@ -182,7 +181,10 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
         const bool tc = tc_pack(dtype, regime, precision, n, k);
         const size_t off = (size_t)round_up((int64_t)pb->bytes, 256);
         const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
-        cudaError_t e = cudaMalloc(&pb->data, tc ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float) : pb->bytes);
+        const bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
+        cudaError_t e = cudaMalloc(&pb->data, tc     ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float)
+                                              : tc64 ? off + tc64_bytes(k, n)
+                                                     : pb->bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             delete pb;
@@ -199,6 +201,11 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
                                        pb->ntiles, static_cast<cudaStream_t>(stream))
                 : launch_pack_b(dtype, k, n, B_dev, ldb, pb->data, pb->kp, pb->w, pb->ntiles,
                                 static_cast<cudaStream_t>(stream));
+        if (e == cudaSuccess && tc64) {
+            pb->tc_data = static_cast<char *>(pb->data) + off;
+            e = launch_pack_b_tc64(k, n, static_cast<const double *>(B_dev), ldb, pb->tc_data,
+                                   static_cast<cudaStream_t>(stream));
+        }
         if (e != cudaSuccess) {
             cudaFree(pb->data);
             delete pb;
@@ -352,23 +359,25 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         }
     } else if (regime == 1) {
         p->np = tall_np(n);
-        p->tc = tc_pack(dtype, regime, precision, n, k);
+        p->tc = tc_pack(dtype, regime, precision, n, k) || tc64_pack(dtype, regime, n, k);
+        // k split in stages of kTallBKS columns; the FP64 guard looks at aligned windows of 64
+        const int64_t stage = p->tc && dtype == TSMM_F64 ? 64 : kTallBKS;
         p->bm = p->tc ? kTcRows : tall_bm(dtype, p->np);
         p->kp = round_up(k, kTallBKS);
         p->slabs = (m + p->bm - 1) / p->bm;
-        const int64_t kstages = p->kp / kTallBKS;
+        const int64_t kstages = (p->kp + stage - 1) / stage;
         // keep the workspace within max_workspace and the grid's y extent legal
         const int64_t per_split = (int64_t)p->np * p->slabs * p->bm * (int64_t)es;
         int64_t max_splits = 65535;
         if (per_split > 0) max_splits = std::min<int64_t>(max_splits, max_workspace / per_split);
-        const int per_sm = p->tc ? 2 : tall_resident_blocks(dtype == TSMM_F64, p->np);
+        const int per_sm = p->tc ? (dtype == TSMM_F64 ? 1 : 2) : tall_resident_blocks(dtype == TSMM_F64, p->np);
         int s = (kstages > 0 && p->slabs > 0)
-                    ? choose_splits(p->slabs, kstages, sms, max_splits, per_sm)
+                    ? choose_splits(p->slabs, kstages, sms, max_splits, per_sm, 4)
                     : 1;
         if (forced_splits > 0)
             s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)forced_splits, kstages, max_splits}));
         const int64_t chunk_stages = kstages > 0 ? (kstages + s - 1) / s : 1;
-        p->kchunk = chunk_stages * kTallBKS;
+        p->kchunk = chunk_stages * stage;
         p->splits = kstages > 0 ? (int)((kstages + chunk_stages - 1) / chunk_stages) : 1;
         if (p->splits > 1) {
             p->workspace_bytes = (size_t)p->splits * (size_t)per_split;
@@ -467,7 +476,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         const cuuint64_t gdim[2] = {(cuuint64_t)m, (cuuint64_t)k};
         const cuuint64_t gstride[1] = {(cuuint64_t)(lda * (int64_t)es)};
         const cuuint32_t box[2] = {(cuuint32_t)p->bm,
-                                   (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k)};
+                                   (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k, p->tc)};
         const cuuint32_t estr[2] = {1, 1};
         CUresult r = encoder()(&p->tmap,
                                p->dtype == TSMM_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -541,7 +550,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
                 const cuuint64_t gdim[2] = {(cuuint64_t)m, (cuuint64_t)k};
                 const cuuint64_t gstride[1] = {(cuuint64_t)(ldd * (int64_t)es)};
                 const cuuint32_t box[2] = {(cuuint32_t)p->bm,
-                                           (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k)};
+                                           (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k, p->tc)};
                 const cuuint32_t estr[2] = {1, 1};
                 const cudaError_t ce = launch_copy_columns(p->dtype, A_dev, lda, m, k, scratch, ldd, s);
                 if (ce == cudaSuccess &&
@@ -578,6 +587,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }
+    if (p->tc && p->dtype == TSMM_F64) return cuda_status(launch_tall_tc64(tma ? &p->tmap : nullptr, a, s));
     if (p->tc) return cuda_status(launch_tall_tc(tma ? &p->tmap : nullptr, a, s));
     cudaError_t e = p->dtype == TSMM_F32 ? launch_tall_f32(tma, p->np, &p->tmap, a, s)
                                          : launch_tall_f64(tma, p->np, &p->tmap, a, s);

@@ -2,6 +2,7 @@
 // bounded waits, and small vector helpers.  Hand-written inline PTX.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 namespace tsmm {
@@ -173,6 +174,15 @@ __device__ __forceinline__ void prefetch_tmap(const void *tmap) {
 // Named barrier over a subset of the block's warps (id 0 is __syncthreads).
 __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// f(std::integral_constant<int, I>{}) for I = B .. E-1, unrolled at compile time.
+template <int B, int E, typename F>
+__device__ __forceinline__ void static_for(F &&f) {
+    if constexpr (B < E) {
+        f(std::integral_constant<int, B>{});
+        static_for<B + 1, E>(f);
+    }
 }
 
 // Vector of N consecutive elements for 16-byte (or smaller) shared/global access.

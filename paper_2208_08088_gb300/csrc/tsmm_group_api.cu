@@ -22,7 +22,8 @@
 namespace tsmm {
 cudaError_t launch_grouped_f32(int np, bool unaligned, int lv, const GroupParams &gp, cudaStream_t s);
 cudaError_t launch_grouped_f64(int np, bool unaligned, int lv, const GroupParams &gp, cudaStream_t s);
-cudaError_t launch_grouped_tc(int width, bool unaligned, const GroupParams &gp, cudaStream_t s);  // tsmm_tall_tc.cu
+cudaError_t launch_grouped_tc(int width, bool unaligned, const GroupParams &gp, cudaStream_t s);    // tsmm_tall_tc.cu
+cudaError_t launch_grouped_tc64(int width, bool unaligned, const GroupParams &gp, cudaStream_t s);  // tsmm_tall_tc64.cu
 }  // namespace tsmm
 
 using namespace tsmm;
@@ -101,7 +102,7 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
         if (kind != 0) {
             const tsmm_plan_t p = items[i].plan;
             if (p->tc) {
-                classes[std::make_tuple((int)p->dtype, (int)tc_width(p->n), kind, kTcForm)].push_back(i);
+                classes[std::make_tuple((int)p->dtype, (int)(p->dtype == TSMM_F64 ? tc64_width(p->n) : tc_width(p->n)), kind, kTcForm)].push_back(i);
                 continue;
             }
             const int lv = kind == 2 ? async_load_variant(p->dtype == TSMM_F32, p->np, items[i].A_dev, items[i].lda)
@@ -136,7 +137,8 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
                 const size_t es = dtype_size(dt);
                 const cuuint64_t gdim[2] = {(cuuint64_t)p->m, (cuuint64_t)p->k};
                 const cuuint64_t gstride[1] = {(cuuint64_t)(it.lda * (int64_t)es)};
-                const cuuint32_t box[2] = {(cuuint32_t)p->bm, (cuuint32_t)kTallBKS};
+                const cuuint32_t box[2] = {(cuuint32_t)p->bm,
+                                           (cuuint32_t)a_box_k(dt, 1, p->precision, p->k, p->tc)};
                 const cuuint32_t estr[2] = {1, 1};
                 if (!unaligned && encoder_grouped()(&g.tmA,
                                       dt == TSMM_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -171,7 +173,8 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
                 total += n_items;
             }
             gp->total_items = total;
-            cudaError_t e = lv == kTcForm    ? launch_grouped_tc(np, unaligned, *gp, s)
+            cudaError_t e = lv == kTcForm    ? (dt == TSMM_F64 ? launch_grouped_tc64(np, unaligned, *gp, s)
+                                                               : launch_grouped_tc(np, unaligned, *gp, s))
                             : dt == TSMM_F32 ? launch_grouped_f32(np, unaligned, lv, *gp, s)
                                              : launch_grouped_f64(np, unaligned, lv, *gp, s);
             if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TSMM_ERR_OUT_OF_MEMORY : TSMM_ERR_CUDA;

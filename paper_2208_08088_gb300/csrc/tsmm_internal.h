@@ -69,6 +69,28 @@ inline bool tc_pack(tsmm_dtype d, int regime, int precision, int64_t n, int64_t 
     return d == TSMM_F32 && regime == 1 && precision == 0 && n > 16 && k > 0;
 }
 
+// FP64 regime (i) on the tensor cores (tsmm_tall_tc64.cuh): steps of kTc64KB columns of k, MMA width per digit.  n = 1 stays
+// with the fma kernel (1.75 ms at m = k = 32768; any n <= 16 takes 1.98 here); k from 256 on, where the truncation of the
+// digits is below the fma chain's rounding (k = 256: 6.6e-17 against 3.9e-16) and the start of a block pays (m = 20000,
+// n = 30, k = 256: 406 us against 54).
+constexpr int kTc64KB = 16;
+constexpr int kTc64Emin = 1023 - 400, kTc64Emax = 1023 + 400;  // range of the scales (exponent fields)
+constexpr int kTc64Guard = 5120, kTc64Windows = 4;
+inline int64_t tc64_width(int64_t n) { return (n + 15) / 16 * 16; }
+// k up to 2^20 keeps the sums' high words below 2^51.
+inline bool tc64_pack(tsmm_dtype d, int regime, int64_t n, int64_t k) {
+    return d == TSMM_F64 && regime == 1 && n > 1 && k >= 256 && k <= (1 << 20);
+}
+// Head of the packed digits of B, in device memory, kTc64Head bytes.  Behind it, for k rounded up to 64: per step of
+// kTc64KB rows 7 digits x width columns, FP16, K-major; then per 64 rows width columns x 64 bytes, the top 7 bits of
+// |b| at the column's scale.
+struct TcB64 {
+    unsigned bad;               // a nonzero column beyond the scales' range, an infinity or a NaN
+    int F[kTallMaxN];           // scale of each column (kTc64Emin: zero column)
+};
+constexpr int kTc64Head = 512;
+static_assert(sizeof(TcB64) <= kTc64Head, "head");
+
 // Load form of the regime (i) kernel for an A that a tensor map cannot describe
 // (its bulk/element-copy kernel): for FP32 widths of 16 and more with A's base
 // 16-byte aligned, lda mod 4 -- every column's offset within 16 bytes is then
@@ -178,6 +200,7 @@ cudaError_t launch_tall_f32(bool tma, int np, const CUtensorMap *tmap, const Tal
 cudaError_t launch_tall_f64(bool tma, int np, const CUtensorMap *tmap, const TallArgs &a,
                             cudaStream_t s);
 
+cudaError_t launch_tall_tc64(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s);
 // The tensor-core kernel; tmap == nullptr: an A that a tensor map cannot describe.
 cudaError_t launch_tall_tc(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s);
 
@@ -199,7 +222,8 @@ constexpr int rank_wide_kc(int64_t k) { return k <= 32 ? 16 : 32; }
 inline bool rank_wide(tsmm_dtype d, int regime, int precision, int64_t k) {
     return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankWideMinK;
 }
-inline int a_box_k(tsmm_dtype d, int regime, int precision, int64_t k) {
+inline int a_box_k(tsmm_dtype d, int regime, int precision, int64_t k, bool tc) {
+    if (tc && d == TSMM_F64) return kTc64KB;
     return rank_wide(d, regime, precision, k) ? rank_wide_kc(k) : kTallBKS;
 }
 // tmC: tensor map of C (box bm x kRankNT) when C meets the TMA rules, else nullptr.
@@ -247,13 +271,16 @@ tsmm_status execute_grouped(const tsmm_group_item *items, int count, tsmm_stream
 // Split-K factor of the regime (i) kernel (planner model in tsmm_api.cu);
 // `resident` = thread blocks per SM.
 int choose_splits(int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits,
-                  int resident = 2);
+                  int resident = 2, int64_t overhead = 4);
 
 cudaError_t launch_pack_b(tsmm_dtype dt, int64_t k, int64_t n, const void *B, int64_t ldb,
                           void *dst, int64_t kp, int64_t w, int64_t ntiles, cudaStream_t s);
 // One launch writes the regime (i) panel and its tensor-core form.
 cudaError_t launch_pack_b_tc(int64_t k, int64_t n, const float *B, int64_t ldb, float *panel, int64_t kp, int np,
                              void *tc_data, float *tc_min, cudaStream_t s);
+// The digits of B behind the panel (tsmm_tall_tc64.cu): bytes of the whole block, and the launches that fill it.
+size_t tc64_bytes(int64_t k, int64_t n);
+cudaError_t launch_pack_b_tc64(int64_t k, int64_t n, const double *B, int64_t ldb, void *dst, cudaStream_t s);
 cudaError_t launch_scale(tsmm_dtype dt, int64_t m, int64_t n, double beta, void *C, int64_t ldc,
                          cudaStream_t s);
 cudaError_t launch_copy_columns(tsmm_dtype dt, const void *src, int64_t lds, int64_t m, int64_t k, void *dst,

@@ -443,15 +443,6 @@ struct AsyncCfg {
     static_assert(Cfg::RESIDENT * (SMEM + 1024) <= 228 * 1024, "resident blocks per SM");
 };
 
-// f(std::integral_constant<int, I>{}) for I = B .. E-1, unrolled at compile time.
-template <int B, int E, typename F>
-__device__ __forceinline__ void static_for(F &&f) {
-    if constexpr (B < E) {
-        f(std::integral_constant<int, B>{});
-        static_for<B + 1, E>(f);
-    }
-}
-
 // An FP32 thread's rows of one stage column whose rows start D elements past
 // the 16-byte-aligned slot start.  rloc and the group stride are multiples of
 // 4, so every group of 4 rows sits D elements past a 16-byte boundary and takes

@@ -20,7 +20,7 @@
 //
 // What the split cannot carry goes another way: a block whose item meets an infinity, a NaN, an overflow (seen as a
 // non-finite sum), or entries so small that a piece of a product could leave FP32's normal range (smallest
-// nonzero |a| times smallest nonzero |b| below 2^-100), recomputes its item with plain fmas (tall_tc_fallback)
+// nonzero |a| times smallest nonzero |b| below 2^-100), recomputes its item with plain fmas (fma_item)
 // before it stores anything, so results follow IEEE fma arithmetic there.
 //
 // Block: one work item = one slab of 128 rows x one k range (the split-K scheme of the fma kernel, same workspace,
@@ -31,6 +31,7 @@
 //   warp 9      tensor-memory owner and MMA issuer;  warp 10  producer of packed B chunks
 #pragma once
 #include "tsmm_internal.h"
+#include "tsmm_fma_item.cuh"
 #include "tsmm_tc.cuh"
 
 namespace tsmm {
@@ -51,7 +52,7 @@ struct TallTcCfg {
     static constexpr int SA = SA_RAW > 6 ? 6 : SA_RAW;
     static constexpr int OFF_B = SA * A_BYTES;
     static constexpr int OFF_BAR = OFF_B + SB * B_BYTES;
-    static constexpr int NBAR = 2 * SA + 2 * SB + 6;
+    static constexpr int NBAR = 2 * SA + 2 * SB + 8;
     static constexpr int SMEM = OFF_BAR + NBAR * 8 + 32;
     static constexpr int PRODUCERS = U ? 2 : 1;
     static constexpr int THREADS = 384;
@@ -60,37 +61,9 @@ struct TallTcCfg {
     static_assert(SA >= 3, "A ring");
     static_assert(COL_A + 96 <= TMEM_COLS, "tensor memory");
     static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two blocks per SM");
-    static_assert(BM * (W / 2) * 4 <= SA * A_BYTES, "fallback exchange");
+    static constexpr int OFF_F = BM * (W / 2) * 4;            // fallback, over the A ring: exchange, then rows of B
+    static_assert(OFF_F + 2 * kFmaRows * W * 4 <= SA * A_BYTES, "fallback");
 };
-
-// Plain fma recomputation of columns [c0, c0 + HW) of one row of the item, from global memory (slow path).
-template <int HW>
-__device__ __forceinline__ void tall_tc_fallback(const TallArgs &a, int64_t row, int64_t k0, int64_t k1, int c0, float *out) {
-    float2 acc[HW / 2];
-#pragma unroll
-    for (int j = 0; j < HW / 2; ++j) acc[j] = make_float2(0.f, 0.f);
-    const bool in = row < a.m;
-    const float *Ap = static_cast<const float *>(a.A) + (in ? row : 0) + k0 * a.lda;
-    const float *Bp = static_cast<const float *>(a.Bp) + k0 * a.np + c0;
-    if (k1 > a.k) k1 = a.k;
-    for (int64_t p = k0; p < k1; ++p, Ap += a.lda, Bp += a.np) {
-        const float x = in ? __ldg(Ap) : 0.f;
-        const float2 x2 = make_float2(x, x);
-#pragma unroll
-        for (int j = 0; j < HW; j += 4) {
-            if (c0 + j < a.np) {
-                const float4 b = __ldg(reinterpret_cast<const float4 *>(Bp + j));
-                acc[j / 2] = __ffma2_rn(x2, make_float2(b.x, b.y), acc[j / 2]);
-                acc[j / 2 + 1] = __ffma2_rn(x2, make_float2(b.z, b.w), acc[j / 2 + 1]);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < HW / 2; ++j) {
-        out[2 * j] = acc[j].x;
-        out[2 * j + 1] = acc[j].y;
-    }
-}
 
 template <int W, bool U>
 __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const TallArgs &a, int64_t slab, int split) {
@@ -105,6 +78,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     uint64_t *conv = bempty + SB;      // [2] pieces of A in tensor memory
     uint64_t *mdone = conv + 2;        // [2] the chunk's MMAs are complete
     uint64_t *drained = mdone + 2;     // [2] accumulator read
+    uint64_t *fbar = drained + 2;      // [2] fallback: rows of B landed
     unsigned *tslot = reinterpret_cast<unsigned *>(bar + Cfg::NBAR);
     unsigned *flag = tslot + 1;
     unsigned *abort_flag = tslot + 2;
@@ -131,6 +105,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
             mbar_init(&conv[b], 4);
             mbar_init(&mdone[b], 1);
             mbar_init(&drained[b], 4);
+            mbar_init(&fbar[b], 1);
         }
         *abort_flag = 0u;
         *unsafe = 0u;
@@ -140,7 +115,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     tcf_before();
     __syncthreads();
     tcf_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);  // uniform: MMA operands stay in uniform registers
 
     if (warp >= 8) {
         reg_dec<40>();
@@ -403,7 +378,9 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
         if (stop) return;  // tile not written; the host sees TSMM_ERR_TIMEOUT
         if (redo) {
             float part[HW];
-            tall_tc_fallback<HW>(a, row, k0, k1, 0, part);
+            fma_item<float, HW>(a, row, k0, k1, 0, part, reinterpret_cast<float *>(smem + Cfg::OFF_F), fbar, abort_flag,
+                                threadIdx.x);
+            if (*abort_flag != 0u) return;
 #pragma unroll
             for (int j = 0; j < HW; ++j) ex[j * BM + r] = part[j];
             named_barrier(1, 256);
@@ -457,7 +434,9 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
     if (stop) return;
     if (redo) {
-        tall_tc_fallback<HW>(a, row, k0, k1, HW, acc + HW);
+        fma_item<float, HW>(a, row, k0, k1, HW, acc + HW, reinterpret_cast<float *>(smem + Cfg::OFF_F), fbar, abort_flag,
+                            threadIdx.x);
+        if (*abort_flag != 0u) return;
         named_barrier(1, 256);
 #pragma unroll
         for (int j = 0; j < HW; ++j) acc[j] = ex[j * BM + r];

@@ -1,0 +1,144 @@
+// Packing, instantiations and launch of the FP64 tensor-core regime (i) kernel.
+#include <cstring>
+
+#include "tsmm_group.cuh"
+#include "tsmm_tall_tc64.cuh"
+
+namespace tsmm {
+
+// Scale of column blockIdx.x: its largest exponent field.
+__global__ void __launch_bounds__(256) pack_b_tc64_scale_kernel(const double *__restrict__ B, int64_t k, int64_t ldb,
+                                                                TcB64 *__restrict__ head) {
+    __shared__ int mx;
+    __shared__ unsigned any;
+    if (threadIdx.x == 0) mx = 0, any = 0u;
+    __syncthreads();
+    const double *col = B + (int64_t)blockIdx.x * ldb;
+    int e = 0;
+    bool nz = false;
+    for (int64_t p = threadIdx.x; p < k; p += 256) {
+        const double x = col[p];
+        e = max(e, (__double2hiint(x) >> 20) & 0x7ff);
+        nz |= x != 0.0;
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (threadIdx.x % 32 == 0) atomicMax(&mx, e);
+    if (nz) any = 1u;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const bool in = mx > kTc64Emin && mx <= kTc64Emax;
+        head->F[blockIdx.x] = in ? mx : kTc64Emin;
+        if (any && !in) atomicOr(&head->bad, 1u);
+    }
+}
+
+// Digits and guard bytes: block = one step of kTc64KB rows, thread = column and pair of rows.
+__global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int64_t n, int64_t ldb, int w,
+                                   unsigned char *__restrict__ base) {
+    const TcB64 *head = reinterpret_cast<const TcB64 *>(base);
+    const int64_t off_guard = kTc64Head + (int64_t)gridDim.x * (7 * w * kTc64KB * 2);
+    unsigned char *dst = base + kTc64Head + blockIdx.x * (int64_t)(7 * w * kTc64KB * 2);
+    for (int e = threadIdx.x; e < w * (kTc64KB / 2); e += blockDim.x) {
+        const int kk = e % (kTc64KB / 2) * 2, j = e / (kTc64KB / 2);
+        const int64_t p = (int64_t)blockIdx.x * kTc64KB + kk;
+        uint32_t hi[2], y0[2], y1[2], g = 0u;
+        const int F = j < n ? head->F[j] : kTc64Emin;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const double x = (p + u < k && j < n) ? B[p + u + (int64_t)j * ldb] : 0.0;
+            hi[u] = (uint32_t)__double2hiint(x);
+            const int s = tc64_shift(tc64_abs(hi[u]), F);
+            const uint64_t y = tc64_fixed(hi[u], (uint32_t)__double2loint(x), s < 0 ? 0 : s);
+            y0[u] = (uint32_t)y;
+            y1[u] = (uint32_t)(y >> 32);
+            const uint64_t x7 = (y - 0x0000808080808080ull) >> 48;
+            g |= (uint32_t)x7 << (8 * u);
+        }
+        const uint32_t sgn = tc64_sign2(hi[0], hi[1]);
+        const uint32_t c = hfma2(sgn, kH1152, 0u);
+        uint32_t d[7];
+        tc64_digits2(y0[0], y0[1], 0x5140, sgn, c, c, d[6], d[5]);
+        tc64_digits2(y0[0], y0[1], 0x7362, sgn, c, c, d[4], d[3]);
+        tc64_digits2(y1[0], y1[1], 0x5140, sgn, c, c, d[2], d[1]);
+        d[0] = hfma2(prmt(prmt(y1[0], y1[1], 0x7362), 0x64646464u, 0x4140), sgn, hfma2(sgn, kH1024, 0u));
+        // digit-major rows (digit i, column j) of 16 k: 8-row groups of 256 bytes
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            const int rw = i * w + j;
+            *reinterpret_cast<uint32_t *>(dst + (rw / 8) * 256 + (kk / 8) * 128 + (rw % 8) * 16 + (kk % 8) * 2) = d[i];
+        }
+        *reinterpret_cast<uint16_t *>(base + off_guard + (p / 64) * (w * 64) + j * 64 + p % 64) = (uint16_t)g;
+    }
+}
+
+size_t tc64_bytes(int64_t k, int64_t n) {
+    const int64_t w = tc64_width(n), steps = round_up(k, 64) / kTc64KB;
+    return (size_t)(kTc64Head + steps * 7 * w * kTc64KB * 2 + round_up(k, 64) * w);
+}
+
+cudaError_t launch_pack_b_tc64(int64_t k, int64_t n, const double *B, int64_t ldb, void *dst, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(dst, 0, sizeof(TcB64), s);
+    if (e != cudaSuccess) return e;
+    pack_b_tc64_scale_kernel<<<(unsigned)n, 256, 0, s>>>(B, k, ldb, static_cast<TcB64 *>(dst));
+    pack_b_tc64_kernel<<<(unsigned)(round_up(k, 64) / kTc64KB), 256, 0, s>>>(B, k, n, ldb, (int)tc64_width(n),
+                                                                           static_cast<unsigned char *>(dst));
+    return cudaGetLastError();
+}
+
+template <int W, bool U>
+static cudaError_t launch_tall_tc64_t(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
+    using Cfg = TallTc64Cfg<W, U>;
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(tall_tc64_kernel<W, U>), Cfg::SMEM);
+    if (e != cudaSuccess) return e;
+    CUtensorMap none;
+    std::memset(&none, 0, sizeof(none));  // U: never read
+    const dim3 grid((unsigned)a.slabs, (unsigned)a.splits);
+    tall_tc64_kernel<W, U><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(U ? none : *tmap, a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tall_tc64(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
+    const bool u = tmap == nullptr;
+    switch (tc64_width(a.n)) {
+        case 16: return u ? launch_tall_tc64_t<16, true>(tmap, a, s) : launch_tall_tc64_t<16, false>(tmap, a, s);
+        case 32: return u ? launch_tall_tc64_t<32, true>(tmap, a, s) : launch_tall_tc64_t<32, false>(tmap, a, s);
+        case 48: return u ? launch_tall_tc64_t<48, true>(tmap, a, s) : launch_tall_tc64_t<48, false>(tmap, a, s);
+        case 64: return u ? launch_tall_tc64_t<64, true>(tmap, a, s) : launch_tall_tc64_t<64, false>(tmap, a, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// Many problems of one MMA width in one launch, one block per work item (tsmm_group.cuh).
+template <int W, bool U>
+__global__ void __launch_bounds__(TallTc64Cfg<W, U>::THREADS, 1)
+    tall_tc64_grouped_kernel(const __grid_constant__ GroupParams gp) {
+    const int64_t item = blockIdx.x;
+    const int p = group_find(gp, item);
+    const TallArgs &a = gp.p[p].a;
+    int64_t slab, split;
+    udivmod(item - gp.p[p].item_begin, a.splits, slab, split);
+    tall_tc64_block<W, U>(&gp.p[p].tmA, a, slab, (int)split);
+}
+
+template <int W, bool U>
+static cudaError_t launch_grouped_tc64_t(const GroupParams &gp, cudaStream_t s) {
+    using Cfg = TallTc64Cfg<W, U>;
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(tall_tc64_grouped_kernel<W, U>), Cfg::SMEM);
+    if (e != cudaSuccess) return e;
+    if (gp.total_items <= 0) return cudaSuccess;
+    if (gp.total_items > INT_MAX) return cudaErrorInvalidValue;
+    tall_tc64_grouped_kernel<W, U><<<(unsigned)gp.total_items, Cfg::THREADS, Cfg::SMEM, s>>>(gp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_grouped_tc64(int width, bool unaligned, const GroupParams &gp, cudaStream_t s) {
+    switch (width) {
+        case 16: return unaligned ? launch_grouped_tc64_t<16, true>(gp, s) : launch_grouped_tc64_t<16, false>(gp, s);
+        case 32: return unaligned ? launch_grouped_tc64_t<32, true>(gp, s) : launch_grouped_tc64_t<32, false>(gp, s);
+        case 48: return unaligned ? launch_grouped_tc64_t<48, true>(gp, s) : launch_grouped_tc64_t<48, false>(gp, s);
+        case 64: return unaligned ? launch_grouped_tc64_t<64, true>(gp, s) : launch_grouped_tc64_t<64, false>(gp, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace tsmm

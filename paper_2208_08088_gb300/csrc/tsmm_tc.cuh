@@ -32,6 +32,15 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a, uint64_t db, u
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
         "r"(a), "l"(db), "r"(idesc), "r"(accumulate));
 }
+// The same with B's descriptor in halves (the address sits in the low one, so steps through a ring are 32-bit additions)
+// and a constant `accumulate`.
+template <bool ACC>
+__device__ __forceinline__ void tc_mma_ts2(uint32_t d, uint32_t a, uint32_t blo, uint32_t bhi, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tmov.b64 b, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}" ::"r"(d),
+        "r"(a), "r"(blo), "r"(bhi), "r"(idesc), "n"(ACC ? 1 : 0));
+}
 // The same with A in shared memory.
 __device__ __forceinline__ void tc_mma_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
