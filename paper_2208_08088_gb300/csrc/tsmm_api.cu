@@ -86,22 +86,59 @@ tsmm_status encode_tmapc(tsmm_plan_t p, void *C_dev, int64_t m, int64_t n, int64
 
 namespace tsmm {
 
-// Split-K choice for regime (i): minimise a wave-quantised time model
-//   T(S) = ceil(slabs*S / resident) * (ceil(kstages / S) + overhead)
-// where `resident` thread blocks run at once (per SM, times the SM count) and
-// `overhead` is the per-block fixed cost (pipeline fill, reduction, epilogue)
-// in stage units.  Smallest S wins ties, which also keeps the workspace small.
-int choose_splits(int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits,
-                  int per_sm, int64_t overhead) {
-    const int64_t resident = (int64_t)per_sm * num_sms;
+// Costs fitted to sweeps of S on GB300 (m 1000..32768, k 500..32768, every kernel; CUDA graphs of 20 calls).  The sum
+// over the partials is the last block's alone and costs as much per split as one to four stages, which a model of
+// waves and stages alone does not see: m = k = 2048, n = 16: 32 splits 23.8 us, 16 16.0, 8 14.5; m = 1024, n = 64,
+// k = 8192: 37 splits 35.5 us, 16 24.1.
+SplitCosts split_costs(tsmm_dtype dt, int np, bool tc, int64_t n) {
+    SplitCosts k{};
+    if (tc && dt == TSMM_F32) {
+        const double w = (double)tc_width(n);
+        k = {2, 0.45, 0.67, kTcRows * kTcKB * 4.0, 3.0, 2.5, 0.35 + 0.00625 * w, 1.0e9};
+    } else if (tc) {
+        const double w = (double)tc64_width(n);
+        k = {1, 1.8 + 0.036 * w, 1.8 + 0.036 * w, kTcRows * 64 * 8.0, 5.0 + 0.12 * w, 2.7 + 0.4 * w, 0.1 + 0.03 * w, 0.0};
+    } else if (dt == TSMM_F32) {
+        const double stage = 0.28 + 0.0015 * np * np;
+        k = {tall_resident_blocks(false, np), stage, stage, tall_block_rows(false, np) * 128.0, 2.5,
+             0.5 + 0.1 * np, 0.03 + 0.031 * np, 64.0e6};
+    } else {  // bound by the FP64 pipe above one column
+        const double stage = np == 1 ? 0.66 : 0.54 * np * 2;
+        k = {tall_resident_blocks(true, np), stage, stage, tall_block_rows(true, np) * 256.0, 2.5,
+             0.5 + 0.05 * np, 0.02 + 0.015 * np, 64.0e6};
+    }
+    return k;
+}
+
+// Split-K choice for regime (i): the S of the least modelled time; the smallest wins ties, which also keeps the
+// workspace small.  Blocks run `resident` to an SM; a stage costs what it does alone, or its share of HBM (7 TB/s) if
+// that is more; a last wave that is not full runs at its own share.  From waves_from bytes of A on, whole waves of
+// stages count at one price: there a block's start and the sum over the partials no longer matter, and HBM's rate needs
+// every SM's full count of blocks (m = k = 32768, n = 16: S = 7 takes 611 us and S = 2 667; n = 64 on the tensor cores:
+// 805 and, at S = 1, 852; but m = 30000, n = 48, k = 3000: S = 5 78 us and S = 1 65).
+int choose_splits(const SplitCosts &k, int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits) {
+    const int64_t resident = (int64_t)k.resident * num_sms;
+    const double bw = 7.0e6;  // bytes per us
+    const bool waves_only = k.waves_from > 0.0 && (double)slabs * (double)kstages * k.bytes >= k.waves_from;
+    auto stage = [&](int64_t blocks) {
+        return std::max(blocks <= num_sms ? k.stage : k.stage2, (double)blocks * k.bytes / bw);
+    };
     int64_t best_s = 1;
     double best_t = -1.0;
     const int64_t s_max = std::max<int64_t>(1, std::min<int64_t>(kstages, max_splits));
     for (int64_t s = 1; s <= s_max; ++s) {
-        const int64_t waves = (slabs * s + resident - 1) / resident;
-        const int64_t per = (kstages + s - 1) / s + overhead;
-        const double t = (double)waves * (double)per;
-        if (best_t < 0 || t < best_t) {
+        const int64_t blocks = slabs * s, per = (kstages + s - 1) / s;
+        const int64_t full = blocks / resident, rem = blocks % resident;
+        const double finish = s > 1 ? k.f0 + k.c * (double)s : 0.0;
+        double t;
+        if (waves_only) {
+            const int64_t waves = full + (rem ? 1 : 0);
+            t = (double)waves * ((double)per + 4.0) * stage(resident) + finish;
+        } else {
+            t = (double)full * ((double)per * stage(resident) + k.block) +
+                (rem ? (double)per * stage(rem) + k.block : 0.0) + finish;
+        }
+        if (best_t < 0 || t < best_t * (1.0 - 1e-9)) {
             best_t = t;
             best_s = s;
         }
@@ -345,8 +382,10 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         const int64_t per_split = (int64_t)p->np * p->slabs * p->bm * (int64_t)es;
         int64_t max_splits = 65535;
         if (per_split > 0) max_splits = std::min<int64_t>(max_splits, max_workspace / per_split);
+        // whole waves of equal stages, a block's start and end worth four of them
+        const SplitCosts x3_costs{1, 1.0, 1.0, 0.0, 4.0, 0.0, 0.0, 0.0};
         int s = (kstages > 0 && p->slabs > 0)
-                    ? choose_splits(p->slabs, kstages, sms, max_splits, 1)
+                    ? choose_splits(x3_costs, p->slabs, kstages, sms, max_splits)
                     : 1;
         if (forced_splits > 0)
             s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)forced_splits, kstages, max_splits}));
@@ -359,7 +398,7 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         }
     } else if (regime == 1) {
         p->np = tall_np(n);
-        p->tc = tc_pack(dtype, regime, precision, n, k) || tc64_pack(dtype, regime, n, k);
+        p->tc = tc_pack(dtype, regime, precision, n, k) || tc64_plan(dtype, regime, m, n, k);
         // k split in stages of kTallBKS columns; the FP64 guard looks at aligned windows of 64
         const int64_t stage = p->tc && dtype == TSMM_F64 ? 64 : kTallBKS;
         p->bm = p->tc ? kTcRows : tall_bm(dtype, p->np);
@@ -370,9 +409,8 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         const int64_t per_split = (int64_t)p->np * p->slabs * p->bm * (int64_t)es;
         int64_t max_splits = 65535;
         if (per_split > 0) max_splits = std::min<int64_t>(max_splits, max_workspace / per_split);
-        const int per_sm = p->tc ? (dtype == TSMM_F64 ? 1 : 2) : tall_resident_blocks(dtype == TSMM_F64, p->np);
         int s = (kstages > 0 && p->slabs > 0)
-                    ? choose_splits(p->slabs, kstages, sms, max_splits, per_sm, 4)
+                    ? choose_splits(split_costs(dtype, p->np, p->tc, n), p->slabs, kstages, sms, max_splits)
                     : 1;
         if (forced_splits > 0)
             s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)forced_splits, kstages, max_splits}));

@@ -207,4 +207,19 @@ __device__ __forceinline__ T ld_cg(const T *p) {
     return __ldcg(p);
 }
 
+// N consecutive elements (16-byte aligned where they fill 16 bytes), L2-coherent.
+template <typename T, int N>
+__device__ __forceinline__ Vec<T, N> ld_cg_vec(const T *p) {
+    Vec<T, N> v;
+    if constexpr (sizeof(T) * N % 16 == 0) {
+#pragma unroll
+        for (int i = 0; i < (int)(sizeof(T) * N / 16); ++i)
+            reinterpret_cast<uint4 *>(v.v)[i] = __ldcg(reinterpret_cast<const uint4 *>(p) + i);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v.v[i] = __ldcg(p + i);
+    }
+    return v;
+}
+
 }  // namespace tsmm

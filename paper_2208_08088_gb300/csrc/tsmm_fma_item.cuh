@@ -91,40 +91,51 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         }
         return true;
     };
-    // up to 8 columns of FP64 (np <= 8 = HW): the halves share the columns and split each stage's rows, and even and odd
-    // rows have sums of their own, which the FP64 pipe's latency asks for (one warp per scheduler with 8 sums ran at 40 %)
-    const bool narrow = sizeof(T) == 8 && HW == 8 && np <= 8;
+    // up to 8 columns of FP64 (np <= 8 = HW): the halves share the columns and split each stage's rows, and 16 sums a
+    // thread (16 / np rows in turn) cover the FP64 pipe's latency, which one warp per scheduler with 8 sums does not (40 %)
     const int half = tid / 128;
-    if (narrow) {
-        FmaAcc<T, HW> acc[2];
-        acc[0].zero();
-        acc[1].zero();
+    auto narrow = [&](auto np_tag) {
+        constexpr int NPW = decltype(np_tag)::value, SETS = 16 / NPW < CH / 2 ? 16 / NPW : CH / 2;
+        FmaAcc<T, NPW> acc[SETS];
+#pragma unroll
+        for (int q = 0; q < SETS; ++q) acc[q].zero();
         T x[CH / 2];
         Ap += (int64_t)(half * (CH / 2)) * a.lda;
 #pragma unroll
         for (int q = 0; q < CH / 2; ++q) x[q] = (in && half * (CH / 2) + q < kk) ? __ldg(Ap + (int64_t)q * a.lda) : T(0);
         for (int c = 0; c < chunks; ++c) {
-            const int b = c & 1;
             stage_wait(c);
             Ap += (int64_t)CH * a.lda;
-            const T *bs = sb + b * CH * np + half * (CH / 2) * np;
+            const T *bs = sb + (c & 1) * CH * NPW + half * (CH / 2) * NPW;
             const int64_t left = kk - (int64_t)(c + 1) * CH - half * (CH / 2);
 #pragma unroll
             for (int q = 0; q < CH / 2; ++q) {
-                acc[q & 1].add(x[q], bs + q * np, np);
+                acc[q % SETS].add(x[q], bs + q * NPW, NPW);
                 x[q] = (in && c + 1 < chunks && q < left) ? __ldg(Ap + (int64_t)q * a.lda) : T(0);
             }
             if (!stage_next(c)) break;
         }
         T *ex = sb + 2 * CH * 16 + tid % 128;
-        if (half == 1) {
+        T s[NPW];
 #pragma unroll
-            for (int j = 0; j < HW; ++j) ex[j * 128] = acc[0].get(j) + acc[1].get(j);
+        for (int j = 0; j < NPW; ++j) {
+            s[j] = acc[0].get(j);
+#pragma unroll
+            for (int q = 1; q < SETS; ++q) s[j] += acc[q].get(j);
+            if (half == 1) ex[j * 128] = s[j];
         }
         named_barrier(1, 256);
 #pragma unroll
-        for (int j = 0; j < HW; ++j) out[j] = half == 0 ? acc[0].get(j) + acc[1].get(j) + ex[j * 128] : T(0);
-        return;
+        for (int j = 0; j < HW; ++j) out[j] = T(0);
+        if (half == 0) {
+#pragma unroll
+            for (int j = 0; j < NPW; ++j) out[j] = s[j] + ex[j * 128];
+        }
+    };
+    if constexpr (sizeof(T) == 8 && HW == 8) {
+        if (np == 2) return narrow(std::integral_constant<int, 2>{});
+        if (np == 4) return narrow(std::integral_constant<int, 4>{});
+        if (np == 8) return narrow(std::integral_constant<int, 8>{});
     }
     FmaAcc<T, HW> acc;
     acc.zero();

@@ -75,14 +75,22 @@ inline bool tc_pack(tsmm_dtype d, int regime, int precision, int64_t n, int64_t 
 // n = 30, k = 256: 406 us against 54).
 constexpr int kTc64KB = 16;
 constexpr int kTc64Emin = 1023 - 400, kTc64Emax = 1023 + 400;  // range of the scales (exponent fields)
-constexpr int kTc64Guard = 5120, kTc64Windows = 4;
+constexpr int kTc64Windows = 8;
+__host__ __device__ constexpr int tc64_guard(int w) { return w <= 48 ? 1200 : 5120; }
 inline int64_t tc64_width(int64_t n) { return (n + 15) / 16 * 16; }
+// Digits of B, and orders of products, per width: eight where tensor memory holds eight accumulators.
+__host__ __device__ constexpr int tc64_digits(int w) { return w <= 48 ? 8 : 7; }
 // k up to 2^20 keeps the sums' high words below 2^51.
 inline bool tc64_pack(tsmm_dtype d, int regime, int64_t n, int64_t k) {
     return d == TSMM_F64 && regime == 1 && n > 1 && k >= 256 && k <= (1 << 20);
 }
+// ... and for at least 64 us of the FP64 pipe: below that a block's start and end weigh as much, and an item that its
+// guard leaves to the fmas has too few blocks beside it (m = 1533, n = 7, k = 605, uneven rows: 28 us, 62 with digits).
+inline bool tc64_plan(tsmm_dtype d, int regime, int64_t m, int64_t n, int64_t k) {
+    return tc64_pack(d, regime, n, k) && (double)m * (double)tall_np(n) * (double)k >= 4.0e7;
+}
 // Head of the packed digits of B, in device memory, kTc64Head bytes.  Behind it, for k rounded up to 64: per step of
-// kTc64KB rows 7 digits x width columns, FP16, K-major; then per 64 rows width columns x 64 bytes, the top 7 bits of
+// kTc64KB rows tc64_digits digits x width columns, FP16, K-major; then per 64 rows width columns x 64 bytes, the top 7 bits of
 // |b| at the column's scale.
 struct TcB64 {
     unsigned bad;               // a nonzero column beyond the scales' range, an infinity or a NaN
@@ -268,10 +276,15 @@ void plan_cache_store(tsmm_dtype dtype, int64_t m, int64_t n, int64_t k, int sms
 // tsmm_execute_grouped (tsmm_group_api.cu), for the server.
 tsmm_status execute_grouped(const tsmm_group_item *items, int count, tsmm_stream_t stream);
 
-// Split-K factor of the regime (i) kernel (planner model in tsmm_api.cu);
-// `resident` = thread blocks per SM.
-int choose_splits(int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits,
-                  int resident = 2, int64_t overhead = 4);
+// Costs of a regime (i) kernel for the choice of its split-K factor, in us: a block's stage of k alone on its SM, its
+// bytes, a block's start and end, and the last block's sum over S partial tiles, f0 + c * S.
+struct SplitCosts {
+    int resident;     // blocks per SM
+    double stage, stage2, bytes, block, f0, c;  // stage2: a stage where the SM has another block
+    double waves_from;  // bytes of A from which whole waves of stages count at one price (0: never)
+};
+SplitCosts split_costs(tsmm_dtype dt, int np, bool tc, int64_t n);
+int choose_splits(const SplitCosts &k, int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits);
 
 cudaError_t launch_pack_b(tsmm_dtype dt, int64_t k, int64_t n, const void *B, int64_t ldb,
                           void *dst, int64_t kp, int64_t w, int64_t ntiles, cudaStream_t s);

@@ -31,6 +31,7 @@
 //   warp 9      tensor-memory owner and MMA issuer;  warp 10  producer of packed B chunks
 #pragma once
 #include "tsmm_internal.h"
+#include "tsmm_finish.cuh"
 #include "tsmm_fma_item.cuh"
 #include "tsmm_tc.cuh"
 
@@ -276,35 +277,14 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
                 c[(int64_t)j * a.ldc] = o;
             }
     };
-    // split-K: the last arriver sums the S partials in the fixed order s = 0..S-1; all 256 threads take part, each one
-    // row and every other group of 8 columns, the loads of four splits in flight together
-    auto finish = [&](int half) {
+    // split-K: take an arrival ticket; the last arriver finishes, all 256 threads of it
+    auto finish = [&]() {
         named_barrier(1, 256);
         if (threadIdx.x == 0) *flag = atomicAdd(a.tickets + slab, 1u) == (unsigned)(a.splits - 1) ? 1u : 0u;
         named_barrier(1, 256);
         if (*flag == 0u) return;
         __threadfence();
-        for (int c0 = half * 8; c0 < n; c0 += 16) {
-            float sum[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sum[j] = 0.f;
-            const float *src = ws + (int64_t)c0 * mpad;
-            for (int sp = 0; sp < a.splits; sp += 4) {
-                float t[4][8];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        t[q][j] =
-                            (sp + q < a.splits && c0 + j < n) ? ld_cg(src + ((int64_t)(sp + q) * a.np + j) * mpad) : 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (sp + q < a.splits) sum[j] += t[q][j];
-            }
-            store(c0, sum, std::integral_constant<int, 8>{});
-        }
+        tc_finish<float, 256>(a, i0, threadIdx.x);
         if (threadIdx.x == 0) a.tickets[slab] = 0u;  // ready for the next launch on this stream
     };
     if (warp < 4) {
@@ -385,7 +365,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
             for (int j = 0; j < HW; ++j) ex[j * BM + r] = part[j];
             named_barrier(1, 256);
         }
-        if (a.splits > 1) finish(0);
+        if (a.splits > 1) finish();
         return;
     }
 
@@ -450,7 +430,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     for (int j = 0; j < W; ++j)
         if (j < n) ws[((int64_t)split * a.np + j) * mpad] = acc[j];
     __threadfence();
-    finish(1);
+    finish();
 }
 
 template <int W, bool U>

@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(256) pack_b_tc64_scale_kernel(const double *__
 __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int64_t n, int64_t ldb, int w,
                                    unsigned char *__restrict__ base) {
     const TcB64 *head = reinterpret_cast<const TcB64 *>(base);
-    const int64_t off_guard = kTc64Head + (int64_t)gridDim.x * (7 * w * kTc64KB * 2);
-    unsigned char *dst = base + kTc64Head + blockIdx.x * (int64_t)(7 * w * kTc64KB * 2);
+    const int64_t off_guard = kTc64Head + (int64_t)gridDim.x * (tc64_digits(w) * w * kTc64KB * 2);
+    unsigned char *dst = base + kTc64Head + blockIdx.x * (int64_t)(tc64_digits(w) * w * kTc64KB * 2);
     for (int e = threadIdx.x; e < w * (kTc64KB / 2); e += blockDim.x) {
         const int kk = e % (kTc64KB / 2) * 2, j = e / (kTc64KB / 2);
         const int64_t p = (int64_t)blockIdx.x * kTc64KB + kk;
@@ -48,24 +48,27 @@ __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int6
             const double x = (p + u < k && j < n) ? B[p + u + (int64_t)j * ldb] : 0.0;
             hi[u] = (uint32_t)__double2hiint(x);
             const int s = tc64_shift(tc64_abs(hi[u]), F);
-            const uint64_t y = tc64_fixed(hi[u], (uint32_t)__double2loint(x), s < 0 ? 0 : s);
+            // one digit more than A: 63 bits below the scale, 0x80 added to the seven low bytes
+            uint64_t m = ((uint64_t)((hi[u] & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x)) << 10;
+            m = s > 63 ? 0ull : m >> (s < 0 ? 0 : s);
+            g |= (uint32_t)(m >> 56) << (8 * u);
+            const uint64_t y = m + 0x0080808080808080ull;
             y0[u] = (uint32_t)y;
             y1[u] = (uint32_t)(y >> 32);
-            const uint64_t x7 = (y - 0x0000808080808080ull) >> 48;
-            g |= (uint32_t)x7 << (8 * u);
         }
         const uint32_t sgn = tc64_sign2(hi[0], hi[1]);
         const uint32_t c = hfma2(sgn, kH1152, 0u);
-        uint32_t d[7];
-        tc64_digits2(y0[0], y0[1], 0x5140, sgn, c, c, d[6], d[5]);
-        tc64_digits2(y0[0], y0[1], 0x7362, sgn, c, c, d[4], d[3]);
-        tc64_digits2(y1[0], y1[1], 0x5140, sgn, c, c, d[2], d[1]);
-        d[0] = hfma2(prmt(prmt(y1[0], y1[1], 0x7362), 0x64646464u, 0x4140), sgn, hfma2(sgn, kH1024, 0u));
+        uint32_t d[8];
+        tc64_digits2(y0[0], y0[1], 0x5140, sgn, c, c, d[7], d[6]);
+        tc64_digits2(y0[0], y0[1], 0x7362, sgn, c, c, d[5], d[4]);
+        tc64_digits2(y1[0], y1[1], 0x5140, sgn, c, c, d[3], d[2]);
+        tc64_digits2(y1[0], y1[1], 0x7362, sgn, c, hfma2(sgn, kH1024, 0u), d[1], d[0]);
         // digit-major rows (digit i, column j) of 16 k: 8-row groups of 256 bytes
 #pragma unroll
-        for (int i = 0; i < 7; ++i) {
+        for (int i = 0; i < 8; ++i) {
             const int rw = i * w + j;
-            *reinterpret_cast<uint32_t *>(dst + (rw / 8) * 256 + (kk / 8) * 128 + (rw % 8) * 16 + (kk % 8) * 2) = d[i];
+            if (i < tc64_digits(w))
+                *reinterpret_cast<uint32_t *>(dst + (rw / 8) * 256 + (kk / 8) * 128 + (rw % 8) * 16 + (kk % 8) * 2) = d[i];
         }
         *reinterpret_cast<uint16_t *>(base + off_guard + (p / 64) * (w * 64) + j * 64 + p % 64) = (uint16_t)g;
     }
@@ -73,7 +76,7 @@ __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int6
 
 size_t tc64_bytes(int64_t k, int64_t n) {
     const int64_t w = tc64_width(n), steps = round_up(k, 64) / kTc64KB;
-    return (size_t)(kTc64Head + steps * 7 * w * kTc64KB * 2 + round_up(k, 64) * w);
+    return (size_t)(kTc64Head + steps * tc64_digits((int)w) * w * kTc64KB * 2 + round_up(k, 64) * w);
 }
 
 cudaError_t launch_pack_b_tc64(int64_t k, int64_t n, const double *B, int64_t ldb, void *dst, cudaStream_t s) {

@@ -10,21 +10,24 @@
 // up: together below 2^-52.7 of 2^E 2^F per term (2^E, 2^F: the powers above the row's and the column's largest
 // entry).  (Splitting a product into exactly accumulated slices: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 2012.)
 //
-// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.44 ms (FP64 pipe 98 % busy before; now 40 TFLOP/s FP64,
-// 2.5 TB/s), n = 4: 7.02 -> 1.98 ms (4.3 TB/s); relative error against 64 bits with compensated sums 2.3e-15 -> 1.2e-16.
+// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.45 ms (FP64 pipe 98 % busy before; now 40 TFLOP/s FP64,
+// 2.5 TB/s), n = 32: 55.7 -> 2.56 ms, n = 4: 7.0 -> 1.98 ms (4.3 TB/s); relative error against compensated sums 1.1e-15 to
+// 2.3e-15 -> 1.0e-16 to 1.2e-16, on rows of very different size (n = 8, k = 2048) 2.6e-16 -> 9.7e-17 (without the eighth
+// digit and order 7: 1.4e-15; they cost nothing up to n = 16 and 11 to 20 % above).
 // Bound by issue: a step of 16 columns costs the converters about 2000 warp instructions (HBM alone would leave 710
-// cycles a step, the MMAs take 900 at n = 64, 260 at n <= 16), and at n = 64 by the drains of the accumulators, which
+// cycles a step, the MMAs take 900 at n = 64, 330 at n <= 16), and at n = 64 by the drains of the accumulators, which
 // tensor memory cannot hold twice there (seven conversions to integers an output had made a drain 4400 cycles; the
-// magic additions below, in one pass: 3.64 -> 3.42 ms).  Two sets of converters, so that one's waits overlap the other's
-// work (n = 4: 2.60 -> 2.31 ms); two sets of digits where they fit (n = 4: 2.22 -> 2.03 ms); a single elected MMA lane
-// (n = 64: 3.97 -> 3.64 ms).
+// magic additions below, in one pass: 3.64 -> 3.42 ms).  Two sets of converters, so that one's waits overlap the
+// other's work (n = 4: 2.60 -> 2.31 ms); two sets of digits where they fit (n = 4: 2.22 -> 2.03 ms); a single elected MMA
+// lane (n = 64: 3.97 -> 3.64 ms).
 //
 // Scale.  E is kept per row and only grows: a chunk with a larger entry closes the current group of chunks (their
 // sums are drained at the old scale) and the 96-bit sums are shifted once.
 //
-// Guard.  The library's bound asks for an error below 4 k 2^-53 sum|a||b|, so the split may be used where sum|a||b| is
-// at least 0.31 * 2^E 2^F; the promoters prove that at the start of the item from the top digits of 64 columns of k
-// (more, if those do not suffice): sum of products of 7-bit digits >= 5120.  Where it cannot be proven (a sparse or
+// Guard.  The library's bound asks for an error below 4 k 2^-53 sum|a||b|, so the split may be used where an item's
+// sum|a||b| is at least 0.07 (W = 64: 0.31) * 2^E 2^F times its share of k; the promoters prove that at the start of the
+// item from the top digits of its first columns (16, and up to 512 while those do not suffice): sum of products of 7-bit
+// digits >= 1200 (5120) times the share.  Where it cannot be proven (a sparse or
 // steeply scaled A or B), and for rows or columns with infinities, NaNs or entries beyond 2^+-400, the block computes
 // its item with FP64 fmas from global memory, which is bound by the FP64 pipe as the fma kernel is.
 //
@@ -35,6 +38,7 @@
 //   warp 16 (and 19: U)  producers of A;  warp 17 tensor memory and MMAs;  warp 18 producer of the digits of B
 #pragma once
 #include "tsmm_internal.h"
+#include "tsmm_finish.cuh"
 #include "tsmm_fma_item.cuh"
 #include "tsmm_tc.cuh"
 
@@ -47,16 +51,18 @@ struct TallTc64Cfg {
     static constexpr int GROUP = 128 / KB;                    // steps per exact group, at most
     static constexpr int A_STRIDE = U ? BM + 4 : BM;          // doubles per column slot
     static constexpr int A_BYTES = KB * A_STRIDE * 8;
-    static constexpr int B_BYTES = 7 * W * KB * 2;            // the digits of a step of B, digit-major
+    static constexpr int ND = tc64_digits(W);                 // digits of B = orders kept = accumulators
+    static constexpr int B_BYTES = ND * W * KB * 2;           // the digits of a step of B, digit-major
     static constexpr int SA = 8, SB = 4;
     static constexpr int OFF_B = SA * A_BYTES;
     static constexpr int OFF_E = OFF_B + SB * B_BYTES;        // row scales of the last ERING steps
     // the guard's digits of B (kTc64Windows windows), later the fallback's rows of B
-    // the promoters read a group's scales when it is complete: converters are then at most 3 steps ahead, with two sets
-    // of accumulators a group more
-    static constexpr int ERING = W == 16 ? 16 : 4;
+    // the promoters read a group's scales once it is complete, when converters may have begun the 4th step after its last
+    // (DB; 3rd otherwise), with two sets of accumulators a group later
+    static constexpr int ERING = W == 16 ? 16 : 8;
     static constexpr int OFF_F = OFF_E + ERING * BM * 4;
-    static constexpr int F_BYTES = W == 16 ? 2 * kFmaRows * W * 8 + 8 * BM * 8 : 2 * kFmaRows * W * 8;
+    static constexpr int F_BYTES = W == 16 ? 2 * kFmaRows * W * 8 + 8 * BM * 8 : kTc64Windows * 64 * W;
+    static_assert(F_BYTES >= 2 * kFmaRows * W * 8, "fallback rows");
     static constexpr int OFF_BAR = OFF_F + F_BYTES;
     static constexpr int NBAR = 2 * SA + 2 * SB + 18;
     static constexpr int SMEM = OFF_BAR + NBAR * 8 + 96;
@@ -65,11 +71,12 @@ struct TallTc64Cfg {
     static constexpr int CREG = W == 64 ? 72 : 80, PREG = W == 64 ? 144 : W == 48 ? 128 : 112;
     static constexpr int MREG = W == 64 ? 48 : W == 48 ? 64 : 96;
     static constexpr int CB = W == 64 ? 4 : 8;                // columns a promoter drains at a time
-    // tensor memory: 7 accumulators of W columns, then the digits of a step of A, 8 columns each: 3-6 (X), 0-2 (Y).
+    static constexpr int SH = W == 64 ? 0 : 4;                // unit of the sums: 2^-SH of the order-5 products
+    // tensor memory: ND accumulators of W columns, then the digits of a step of A, 8 columns each: 3-6 (X), 0-2 (Y).
     // DB: two sets of digits, by step parity; else one, whose X and Y parts are refilled in turn
     static constexpr bool DB = W <= 48;
     static constexpr bool DDB = W == 16;                      // two sets of accumulators, by group parity
-    static constexpr int COL_X = (DDB ? 14 : 7) * W, COL_Y = COL_X + 32, COL_SET = DB ? 56 : 0;
+    static constexpr int COL_X = (DDB ? 2 : 1) * ND * W, COL_Y = COL_X + 32, COL_SET = DB ? 56 : 0;
     static constexpr int TMEM_COLS = 512;
     static_assert(256 * CREG + 256 * PREG + 128 * MREG <= THREADS * 96, "register split");
     static_assert(COL_Y + 24 + COL_SET <= TMEM_COLS, "tensor memory");
@@ -329,7 +336,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                     const uint32_t set = tmem + (u & 1) * Cfg::COL_SET;
                     static_for<I0, I1>([&](auto i_tag) {
                         constexpr int i = decltype(i_tag)::value;
-                        static_for<0, 7 - i>([&](auto j_tag) {
+                        static_for<0, Cfg::ND - i>([&](auto j_tag) {
                             constexpr int j = decltype(j_tag)::value;
                             const uint32_t at = set + (i >= 3 ? Cfg::COL_X + (i - 3) * 8 : Cfg::COL_Y + i * 8);
                             tc_mma_ts2<!(fresh && (i == 3 || (i == 0 && j < 3)))>(acc + (uint32_t)((i + j) * W), at,
@@ -358,7 +365,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                         fresh = true;
                         cnt = 0;
                         ++g;
-                        acc = tmem + (Cfg::DDB ? (uint32_t)(g & 1) * (7 * W) : 0u);
+                        acc = tmem + (Cfg::DDB ? (uint32_t)(g & 1) * (Cfg::ND * W) : 0u);
                     }
                     ++cnt;
                     if (fresh) mmas(u_tag, c3, c7, std::true_type{});
@@ -406,6 +413,17 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     const int r = threadIdx.x % BM;
     const int64_t row = i0 + r;
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    // split-K: take an arrival ticket; the last arriver finishes, its converters and promoters
+    auto finish = [&]() {
+        named_barrier(3, 512);
+        if (threadIdx.x == 0)  // an item given up in its fallback takes no ticket
+            *flag = *abort_flag == 0u && atomicAdd(a.tickets + slab, 1u) == (unsigned)(a.splits - 1) ? 1u : 0u;
+        named_barrier(3, 512);
+        if (*flag == 0u) return;
+        __threadfence();
+        tc_finish<double, 512>(a, i0, threadIdx.x);
+        if (threadIdx.x == 0) a.tickets[slab] = 0u;  // ready for the next launch on this stream
+    };
     if (warp < 8) {
         // ---------------------------------------------------- converters
         reg_dec<Cfg::CREG>();
@@ -520,6 +538,8 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             atomicOr(abort_flag, 1u);
         }
         named_barrier(1, 512);  // the promoters read the last scales after it
+        if (*abort_flag != 0u || a.splits == 1) return;
+        finish();
         return;
     }
 
@@ -532,6 +552,8 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     bool ok = true;
 
     // guard: a lower bound of sum|a||b| over the row, column by column, in units of 2^-14 2^E0 2^F
+    // The item's share of the bound, 4 k 2^-53 of its own sum|a||b|, against its error, k_item 2^-54.9 (2^-52.7) 2^E 2^F:
+    const int need = (int)((k1 - k0) * tc64_guard(W) / a.k) + 1;
     int E0 = 0, bound = 0x7fffffff;
     const unsigned bad_b = tb->bad;  // a column of B that the digits cannot hold
     uint32_t fzero = 0u;             // columns that do not count: zero, or beyond n
@@ -577,10 +599,14 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             for (int j = 0; j < HW; ++j)
                 if (!(fzero >> j & 1u)) bound = min(bound, (int)sum[j]);
             if (row >= a.m) bound = 0x7fffffff;
-            if (__all_sync(0xffffffffu, bound >= 4 * kTc64Guard)) break;
+            if (__all_sync(0xffffffffu, bound >= 4 * need)) break;
+            // no more than half of what is needed in sight: given up (a block of columns takes about a microsecond)
+            if (q16 >= 3 && __any_sync(0xffffffffu, (int64_t)bound * min(kTc64Windows * 4, (int)((k1 - k0) / 16)) <
+                                                        (int64_t)(need / 2) * (q16 + 1)))
+                break;
         }
         release_reads_to_async_copy();  // the fallback's copies may follow
-        if (bound < kTc64Guard) {
+        if (bound < need) {
             // too small: fmas, unless the row is zero throughout
             const uint64_t *rp = static_cast<const uint64_t *>(a.A) + row;
             uint64_t any = 0;
@@ -594,7 +620,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     if (lane == 0) mbar_arrive(verdict);
     const bool started = __all_sync(0xffffffffu, ok && go());
 
-    // sums of 96 bits per output, in units of the order-5 products
+    // sums of 96 bits per output
     int64_t vh[HW];
     uint32_t vl[HW];
 #pragma unroll
@@ -628,17 +654,18 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                 vl[j] = l;
             }
         }
-        // V += 2^32 (D1 + 2^8 D0) + 2^24 D2 + 2^16 D3 + 2^8 D4 + (D5 + 2^-8 D6), in units of the order-5 products.  Conversions
-        // to integers take the XU pipe 8 cycles each, so only the sums that need all their 24 bits go there (D2, D3,
-        // D4); D0 and D1 stay within 2^22 and take a magic addition, D5 + 2^-8 D6 one that rounds to a multiple of 4 (by
-        // 2^-53 of 2^E 2^F at most, once a group).  All seven conversions: 3600 cycles a group at W = 64.
-        constexpr int CB = Cfg::CB;
+        // V += 2^SH (2^40 D0 + 2^32 D1 + 2^24 D2 + 2^16 D3 + 2^8 D4 + D5 + 2^-8 D6 + 2^-16 D7).
+        // A conversion to integers takes the XU pipe 8 cycles, so only sums that need their 24 bits go there;
+        // D0 and D1 stay within 2^22 and take a magic addition, and so does at seven orders D5 + 2^-8 D6, rounded to a
+        // multiple of 4 (by 2^-53 of 2^E 2^F at most, once a group).  With all seven converted a drain took 4400 cycles
+        // at W = 64.
+        constexpr int CB = Cfg::CB, SH = Cfg::SH;
         constexpr uint32_t kM23 = 0x4b400000u, kM25 = 0x4c400000u;  // 1.5 * 2^23, 1.5 * 2^25
-        const uint32_t acc0 = tlane + (Cfg::DDB ? (uint32_t)(g & 1) * (7 * W) : 0u) + c0;
+        const uint32_t acc0 = tlane + (Cfg::DDB ? (uint32_t)(g & 1) * (Cfg::ND * W) : 0u) + c0;
 #pragma unroll
         for (int c = 0; c < HW; c += CB) {
-            uint32_t d[7][CB];
-            tc_ldn<7, CB>(acc0 + c, W, d);
+            uint32_t d[Cfg::ND][CB];
+            tc_ldn<Cfg::ND, CB>(acc0 + c, W, d);
             if (c + CB == HW) {
                 tcf_before();
                 __syncwarp();
@@ -646,16 +673,20 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             }
 #pragma unroll
             for (int j = 0; j < CB; ++j) {
-                const float t = fmaf(__uint_as_float(d[6][j]), 0.00390625f, __uint_as_float(d[5][j]));
-                const int i56 = (int)(__float_as_uint(t + __uint_as_float(kM25)) - kM25);
-                int64_t L = (int64_t)(uint64_t)vl[c + j] + (int64_t)i56 * 4;
-                L += (int64_t)__float2int_rn(__uint_as_float(d[4][j])) * 256;
-                L += (int64_t)__float2int_rn(__uint_as_float(d[3][j])) * 65536;
-                L += (int64_t)__float2int_rn(__uint_as_float(d[2][j])) * 16777216;
+                float t = __uint_as_float(d[6][j]);
+                if constexpr (Cfg::ND == 8) t = fmaf(__uint_as_float(d[7][j]), 0.00390625f, t);
+                t = fmaf(t, 0.00390625f, __uint_as_float(d[5][j]));
+                int64_t L = (int64_t)(uint64_t)vl[c + j];
+                if constexpr (Cfg::ND == 8) L += __float2int_rn(t * 16.f);
+                else L += (int64_t)(int)(__float_as_uint(t + __uint_as_float(kM25)) - kM25) * 4;
+                L += (int64_t)__float2int_rn(__uint_as_float(d[4][j])) * (1 << (8 + SH));
+                L += (int64_t)__float2int_rn(__uint_as_float(d[3][j])) * (1 << (16 + SH));
+                L += (int64_t)__float2int_rn(__uint_as_float(d[2][j])) * (1 << (24 + SH));
                 vl[c + j] = (uint32_t)L;
                 const uint32_t h = __float_as_uint(__uint_as_float(d[0][j]) + __uint_as_float(kM23)) * 256u +
-                                   __float_as_uint(__uint_as_float(d[1][j]) + __uint_as_float(kM23));
-                vh[c + j] += (int64_t)((int)(L >> 32) + (int)(h - kM23 * 257u));
+                                   __float_as_uint(__uint_as_float(d[1][j]) + __uint_as_float(kM23)) - kM23 * 257u;
+                if constexpr (SH == 0) vh[c + j] += (int64_t)((int)h + (int)(L >> 32));
+                else vh[c + j] += (int64_t)(int)h * (1 << SH) + (L >> 32);
             }
         }
         if (slot & 64u) break;
@@ -668,7 +699,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         // infinities and NaNs, rows wholly below the scales, and a row that grew after its guard columns
         const int sft = E - E0;
         if (E > kTc64Emax || (E == kTc64Emin && bound != 0x7fffffff) ||
-            (bound != 0x7fffffff && (sft > 30 || (bound >> max(sft, 0)) < kTc64Guard)))
+            (bound != 0x7fffffff && (sft > 30 || (bound >> max(sft, 0)) < need)))
             *unsafe = 1u;
     }
     tcf_before();
@@ -680,9 +711,13 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     if (redo) {
         fma_item<double, HW>(a, row, k0, k1, c0, acc, reinterpret_cast<double *>(smem + Cfg::OFF_F), fbar, abort_flag,
                              threadIdx.x - 256);
-        if (*abort_flag != 0u) return;
+        if (*abort_flag != 0u) {
+            if (a.splits > 1) finish();  // the converters wait there
+            return;
+        }
     } else {
-        // |x| = X 2^(E-1077), an order-5 product has weight 2^56; the sums stay below 2^51 * 2^32.  The upper 64 bits of the
+        // |x| = X 2^(E-1077) with digits of weight 2^(48-8i); an order-5 product has weight 2^56 and the sums' unit 2^-SH of it.
+        // They stay below 2^55 * 2^32.  The upper 64 bits of the
         // magnitude are rounded to a double, whose exponent and sign are then set by integer operations (FP64
         // arithmetic on 128 x W values would take longer than a group of MMAs)
 #pragma unroll
@@ -698,7 +733,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             const int sh = max(0, 32 - __clzll((long long)h));
             const uint64_t u = h << (32 - sh) | l >> sh;
             const double d = __ull2double_rn(u);
-            const uint32_t hw = (uint32_t)__double2hiint(d) + (uint32_t)((sh + E + F - 2154 + 56) * 1048576);
+            const uint32_t hw = (uint32_t)__double2hiint(d) + (uint32_t)((sh + E + F - 2154 + 56 - Cfg::SH) * 1048576);
             acc[j] = u == 0ull ? 0.0 : __hiloint2double((int)(hw | sg), __double2loint(d));
         }
     }
@@ -731,31 +766,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     for (int j = 0; j < HW; ++j)
         if (c0 + j < n) ws[((int64_t)split * a.np + c0 + j) * mpad] = acc[j];
     __threadfence();
-    named_barrier(1, 256);
-    if (threadIdx.x == 256) *flag = atomicAdd(a.tickets + slab, 1u) == (unsigned)(a.splits - 1) ? 1u : 0u;
-    named_barrier(1, 256);
-    if (*flag == 0u) return;
-    __threadfence();
-    // last arriver: the S partials summed in the fixed order s = 0..S-1, the loads of four splits in flight together
-    for (int c = half * 4; c < n; c += 8) {
-        double sum[4] = {0.0, 0.0, 0.0, 0.0};
-        const double *src = ws + (int64_t)c * mpad;
-        for (int sp = 0; sp < a.splits; sp += 4) {
-            double t[4][4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    t[q][j] = (sp + q < a.splits && c + j < n) ? ld_cg(src + ((int64_t)(sp + q) * a.np + j) * mpad) : 0.0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (sp + q < a.splits) sum[j] += t[q][j];
-        }
-        store(c, sum, std::integral_constant<int, 4>{});
-    }
-    if (threadIdx.x == 256) a.tickets[slab] = 0u;  // ready for the next launch on this stream
+    finish();
 }
 
 template <int W, bool U>

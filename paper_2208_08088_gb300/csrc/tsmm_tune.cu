@@ -165,12 +165,16 @@ tsmm_status tsmm_autotune(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, con
     // candidate split counts: the model's choice for 1..4 resident blocks per
     // SM, its halves and doubles, no split, and counts that fill whole waves
     std::set<int64_t> cand;
-    for (int per_sm = 1; per_sm <= 4; ++per_sm)
-        cand.insert(choose_splits(base->slabs, kstages, sms, kstages, per_sm));
+    SplitCosts costs = split_costs(dtype, base->np, base->tc, n);
+    const int resident = costs.resident;
+    for (int per_sm = 1; per_sm <= 4; ++per_sm) {
+        costs.resident = per_sm;
+        cand.insert(choose_splits(costs, base->slabs, kstages, sms, kstages));
+    }
     const int64_t h = base->splits;
     for (int64_t c : {h, h / 2, 2 * h, (int64_t)1}) cand.insert(c);
     for (int waves = 1; waves <= 4; ++waves) {
-        const int64_t want = (int64_t)waves * tall_resident_blocks(dtype == TSMM_F64, base->np) * sms;
+        const int64_t want = (int64_t)waves * resident * sms;
         cand.insert(std::max<int64_t>(1, want / std::max<int64_t>(1, base->slabs)));
     }
     std::vector<int64_t> cands;

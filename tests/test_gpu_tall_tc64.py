@@ -7,19 +7,28 @@ import pytest
 import torch
 
 import paper_2208_08088_gb300 as tsmm
-import tsmm_inputs as ti
 from gpu_util import assert_parity, run, to_device
 
 pytestmark = pytest.mark.gpu
 
 
 def gen(m, n, k, dist="uniform"):
-    return tuple(ti.matrix_np(r, c, s, dist, np.float64) for r, c, s in ((m, k, 31), (k, n, 32), (m, n, 33)))
+    rng = np.random.default_rng(31)
+    draw = (lambda r, c: rng.uniform(-1, 1, (c, r)).T) if dist == "uniform" else \
+        (lambda r, c: rng.integers(-4, 5, (c, r)).astype(np.float64).T)
+    return draw(m, k), draw(k, n), draw(m, n)
+
+
+def rows_for(n, k, extra):
+    """The fewest rows that the digits serve (m * padded n * k >= 4e7), and a few more."""
+    np_ = next(w for w in (2, 4, 8, 16, 24, 32, 48, 64) if w >= n)
+    return -(-40_000_000 // (np_ * k)) + extra
 
 
 @pytest.mark.parametrize("n", [2, 15, 17, 33, 48, 64])
-@pytest.mark.parametrize("m,k,pad", [(1, 256, 0), (127, 257, 1), (129, 319, 0), (300, 1025, 3), (2305, 4100, 1)])
-def test_widths_and_edges(m, n, k, pad):
+@pytest.mark.parametrize("extra,k,pad", [(0, 256, 0), (1, 257, 1), (63, 319, 0), (130, 1025, 3), (5, 4100, 1)])
+def test_widths_and_edges(extra, n, k, pad):
+    m = rows_for(n, k, extra)
     A, B, C0 = gen(m, n, k)
     C, pl, _ = run(A, B, C0, -1.25, 0.75, lda=m + pad)
     assert pl.info()["bm"] == 128
@@ -29,12 +38,14 @@ def test_widths_and_edges(m, n, k, pad):
     assert_parity(C, A, B, C0, 1.5, 0.5, exact=True)
 
 
-@pytest.mark.parametrize("lda", [300, 301])
+@pytest.mark.parametrize("pad", [0, 1])
 @pytest.mark.parametrize("n", [4, 30, 64])
-def test_growing_rows_are_exact(n, lda):
+def test_growing_rows_are_exact(n, pad):
     """Entries grow along k by powers of two, at other places in every row: scales grow in mid-group, sums are shifted.
     Integers below 2^21 against integers below 16: every sum exact."""
-    m, k = 300, 900
+    k = 900
+    m = rows_for(n, k, 6) // 2 * 2
+    lda = m + pad
     rng = np.random.default_rng(5)
     A = rng.integers(-8, 9, size=(m, k)).astype(np.float64)
     for i in range(m):
@@ -50,7 +61,8 @@ def test_growing_rows_are_exact(n, lda):
 @pytest.mark.parametrize("dist", ["normal", "lognormal", "sparse", "identity", "zero_rows", "triangular"])
 def test_distributions_within_bound(dist, n):
     """What the guard proves and what it hands to the fmas (single products stay exact: identity)."""
-    m, k = 260, 700
+    k = 700
+    m = rows_for(n, k, 3)
     rng = np.random.default_rng(8)
     A = rng.standard_normal((m, k))
     B = rng.standard_normal((k, n))
@@ -67,7 +79,7 @@ def test_distributions_within_bound(dist, n):
         A[::3] = 0.0
         B[:, 0] = 0.0
     elif dist == "triangular":
-        A *= np.arange(k)[None, :] >= 2 * np.arange(m)[:, None]
+        A *= np.arange(k)[None, :] >= 2 * (np.arange(m)[:, None] % 350)
     A, B = np.asfortranarray(A), np.asfortranarray(B)
     C, _, _ = run(A, B, None, 1.0, 0.0)
     if dist == "identity":
@@ -75,13 +87,13 @@ def test_distributions_within_bound(dist, n):
     assert_parity(C, A, B, None, 1.0, 0.0)
 
 
-@pytest.mark.parametrize("lda", [300, 301])
+@pytest.mark.parametrize("pad", [0, 1])
 @pytest.mark.parametrize("what", ["inf_a", "nan_a", "inf_b", "huge", "tiny_a", "tiny_b", "subnormal"])
 @pytest.mark.parametrize("n,k", [(5, 700), (64, 5000)])
-def test_values_the_digits_cannot_carry(what, n, k, lda):
-    m = 300
+def test_values_the_digits_cannot_carry(what, n, k, pad):
+    m = rows_for(n, k, 300) // 2 * 2
+    lda = m + pad
     A, B, C0 = (x.copy(order="F") for x in gen(m, n, k, "integer"))
-    exact = True
     if what == "inf_a":
         A[140, k - 1] = np.inf
     elif what == "nan_a":
@@ -104,7 +116,7 @@ def test_values_the_digits_cannot_carry(what, n, k, lda):
 
 def test_grouped_widths_equal_single_launches():
     items, single, outs = [], [], []
-    for i, (m, n, k, pad) in enumerate([(500, 2, 300, 0), (1000, 16, 2000, 1), (129, 40, 256, 1), (700, 48, 999, 0),
+    for i, (m, n, k, pad) in enumerate([(9000, 2, 3000, 0), (1300, 16, 2000, 1), (3300, 40, 256, 1), (900, 48, 999, 0),
                                         (2000, 64, 3000, 0), (333, 63, 5000, 1), (64, 16, 128, 0), (200, 1, 900, 0)]):
         A, B, C0 = gen(m, n, k)
         if i == 3:
