@@ -42,8 +42,9 @@
  *     |A[i,p]||B[p,j]| + |beta||C0[i,j]|) with u = 2^-24 (F32) / 2^-53 (F64).
  *     Products are accumulated with IEEE fma in the working precision, or on the
  *     tensor cores from splits of every entry (errors measured smaller than the
- *     fma chain's): F32 with 16 < n <= 64 from exact splits into three BF16
- *     values with all products down to 2^-25 of |a||b|; F64 with 1 < n <= 64 and
+ *     fma chain's): F32 with 16 < n <= 64, or with n > 64 and k > 32, from exact
+ *     splits into three BF16 values with all products down to 2^-25 of |a||b|;
+ *     F64 with 1 < n <= 64 and
  *     256 <= k <= 2^20 from 56-bit fixed point cut into seven 8-bit digits whose
  *     products are summed exactly.  Inputs such a split cannot carry within the
  *     bound (infinities, NaNs, overflow, extreme or very unevenly scaled

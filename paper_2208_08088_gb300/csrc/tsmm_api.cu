@@ -219,8 +219,10 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
         const size_t off = (size_t)round_up((int64_t)pb->bytes, 256);
         const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
         const bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
+        const bool rtc = rank_tc(dtype, regime, precision, k);
         cudaError_t e = cudaMalloc(&pb->data, tc     ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float)
                                               : tc64 ? off + tc64_bytes(k, n)
+                                              : rtc  ? off + rank_tc_bytes(k, pb->ntiles)
                                                      : pb->bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -238,6 +240,11 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
                                        pb->ntiles, static_cast<cudaStream_t>(stream))
                 : launch_pack_b(dtype, k, n, B_dev, ldb, pb->data, pb->kp, pb->w, pb->ntiles,
                                 static_cast<cudaStream_t>(stream));
+        if (e == cudaSuccess && rtc) {
+            pb->tc_data = static_cast<char *>(pb->data) + off;
+            e = launch_pack_b_rank_tc(k, n, static_cast<const float *>(B_dev), ldb, pb->ntiles, pb->tc_data,
+                                      static_cast<cudaStream_t>(stream));
+        }
         if (e == cudaSuccess && tc64) {
             pb->tc_data = static_cast<char *>(pb->data) + off;
             e = launch_pack_b_tc64(k, n, static_cast<const double *>(B_dev), ldb, pb->tc_data,
@@ -541,6 +548,8 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
             ra.kp = pb->kp;
             ra.A = A_dev;
             ra.Bp = pb->data;
+            ra.Bt = nullptr;
+            ra.bmin = nullptr;
             ra.C = C_dev;
             ra.alpha = alpha;
             ra.beta = beta;
@@ -568,6 +577,8 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         ra.kp = pb->kp;
         ra.A = A_dev;
         ra.Bp = pb->data;
+        ra.Bt = pb->tc_data;
+        ra.bmin = nullptr;
         ra.C = C_dev;
         ra.alpha = alpha;
         ra.beta = beta;
@@ -610,18 +621,21 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
                 scratch = nullptr;
             }
         }
+        const bool rtc = tma_a && rank_tc(p->dtype, p->regime, p->precision, k);
         // C tiles by TMA (C0 prefetch; C0 and C in the FP32 k > 32 kernel): the
         // same 16-byte rules for C
         const bool tmc = tma_a && c_tma_ok(C_dev, ldc, n, es);
         if (tmc) {
-            const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, kRankNT);
+            const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, rtc ? kRankTcSub : kRankNT);
             if (st != TSMM_OK) {
                 if (scratch) cudaFreeAsync(scratch, s);
                 return st;
             }
         }
-        const cudaError_t e = launch_rankk(p->dtype, tma_a ? (scratch ? &tm_scratch : &p->tmap) : nullptr,
-                                           tmc ? &p->tmapc : nullptr, ra, p->status, s);
+        const CUtensorMap *ta = tma_a ? (scratch ? &tm_scratch : &p->tmap) : nullptr;
+        const CUtensorMap *tc = tmc ? &p->tmapc : nullptr;
+        const cudaError_t e = rtc ? launch_rankk_tc(ta, tc, ra, p->status, s)
+                                  : launch_rankk(p->dtype, ta, tc, ra, p->status, s);
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }

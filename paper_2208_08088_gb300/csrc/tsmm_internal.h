@@ -219,21 +219,33 @@ struct RankArgs {
     void *C;
     double alpha, beta;
     int num_sms;     // persistent grid size = resident blocks x SMs
+    const void *Bt;         // tensor-core form of B, and the smallest magnitudes in its chunks
+    const uint32_t *bmin;
 };
 // tmA: tensor map of A (box bm x 32) or nullptr for the plain-load kernel;
-// The FP32 regime (ii) kernel for k >= kRankWideMinK streams k in chunks of
-// rank_wide_kc(k): 16 up to k = 32 (three blocks per SM), 32 above (two blocks
-// per SM), so that every tile has at least two chunks.  Its A tensor map box is
-// bm x rank_wide_kc(k); every other kernel's is bm x kTallBKS.
+// The FP32 regime (ii) kernel for k in kRankWideMinK..32 streams k in chunks of kRankWideKC, so its A
+// tensor map's box is bm x kRankWideKC; every other kernel's is bm x kTallBKS.  From kRankTcMinK on the
+// tensor cores serve it (tsmm_rankk_tc.cu; tmC with a box of bm x kRankTcSub): at m = n = 16384, beta = 1,
+// the wide kernel in chunks of 32 took 0.414 / 0.566 / 1.063 ms at k = 40 / 64 / 128, they take 0.365 / 0.355 /
+// 0.369; at k = 32 the wide kernel's 0.35 is already the output stream's.
 constexpr int kRankWideMinK = 17;
-constexpr int rank_wide_kc(int64_t k) { return k <= 32 ? 16 : 32; }
+constexpr int kRankWideKC = 16;
+constexpr int kRankTcMinK = 33;
+constexpr int kRankTcSub = 32;
+inline bool rank_tc(tsmm_dtype d, int regime, int precision, int64_t k) {
+    return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankTcMinK;
+}
 inline bool rank_wide(tsmm_dtype d, int regime, int precision, int64_t k) {
-    return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankWideMinK;
+    return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankWideMinK && k < kRankTcMinK;
 }
 inline int a_box_k(tsmm_dtype d, int regime, int precision, int64_t k, bool tc) {
     if (tc && d == TSMM_F64) return kTc64KB;
-    return rank_wide(d, regime, precision, k) ? rank_wide_kc(k) : kTallBKS;
+    return rank_wide(d, regime, precision, k) ? kRankWideKC : kTallBKS;
 }
+size_t rank_tc_bytes(int64_t k, int64_t ntiles);
+cudaError_t launch_pack_b_rank_tc(int64_t k, int64_t n, const float *B, int64_t ldb, int64_t ntiles, void *dst, cudaStream_t s);
+cudaError_t launch_rankk_tc(const CUtensorMap *tmA, const CUtensorMap *tmC, const RankArgs &a, unsigned *status,
+                            cudaStream_t s);
 // tmC: tensor map of C (box bm x kRankNT) when C meets the TMA rules, else nullptr.
 cudaError_t launch_rankk(tsmm_dtype dt, const CUtensorMap *tmA, const CUtensorMap *tmC,
                          const RankArgs &a, unsigned *status, cudaStream_t s);

@@ -494,41 +494,31 @@ __global__ void __launch_bounds__(256, 2) rankk_plain_kernel(const RankArgs a, b
     ep.template store<LVC>(acc, a, i0, tile, tm, tn, ealpha, ebeta);
 }
 
-// FP32, k > 32 (FMA-bound).  A 16-byte shared-memory load costs
+// FP32, k = 17..32 (above, the tensor cores: tsmm_rankk_tc.cu).  A 16-byte shared-memory load costs
 // four wavefronts whatever its address pattern, and the SM serves one per
 // cycle; the 8 x 4 register tiles above need 1.5 per cycle at the FMA peak,
 // so this kernel uses 8 x 8 tiles (1.0 per cycle): 4 consumer warps own the
 // same 128 x 64 C tile as a 2 x 2 grid of 64 x 32 warp tiles, lane
 // (lm = lane % 8, ln = lane / 8) owning rows {wm*64 + lm*4 + r, +32} and
 // columns {wn*32 + ln*4 + c, +16} (r, c < 4); a warp's A reads cover one
-// 128-byte line, its B reads 64 bytes.  For k > 32, k streams in chunks of 32
-// through 3 stages (24 KB each) and the C tile has one 32 KB buffer: two blocks
-// (8 consumer warps) per SM, each chunk unrolled whole.  Chunks of 16 (3 stages
-// of 12 KB) fit three blocks per SM, but each chunk's wait and release costs a
-// fixed stretch of issue: their main loop ran at ~0.72 of the FMA peak against
-// ~0.79 for chunks of 32.  For k in 17..32 the chunks of 16 stay (two chunks
-// per tile, so the C0 copy overlaps the second).
+// 128-byte line, its B reads 64 bytes.  k streams in two chunks of 16 per tile
+// through 3 stages (12 KB each; three blocks per SM with the 32 KB C tile), so
+// the C0 copy overlaps the second.
 //
 // TMA_EPI (C meets the TMA rules): the producer brings the C0 tile into the
 // buffer with one tensor copy while the tile's products run; the epilogue
 // overwrites it in place with alpha*acc + beta*C0.  The producer then writes it
 // out with a TMA store and, once the store has read the buffer, issues the next
-// tile's C0 copy into it -- from the next tile's second chunk on, so the copy has
-// that tile's chunks to land (without it, the copy issued one chunk before the
-// epilogue was still in flight at half of the k = 64 epilogues).  With beta = 1
-// and k > 32 there is no C0 copy: the epilogue writes alpha*acc into the buffer and the
-// producer adds it to C with a TMA reduce-add (cp.reduce.async.bulk.tensor
-// .add), which reads C0 and writes C in L2 -- the same single rounding of
-// C0 + alpha*acc as the fma(1, C0, alpha*acc) of the other form -- so the tile
-// never waits for C0.
+// tile's C0 copy into it.  (A TMA reduce-add into C instead of the C0 copy
+// streamed slower: 0.43 vs 0.35 ms at m = n = 16384, k = 32, beta = 1.)
 // Otherwise the epilogue moves C0 and C with 16-byte loads and stores.
 namespace {
-template <bool TMA_EPI, int KC_>
+template <bool TMA_EPI>
 struct WideCfg {
     static constexpr int BMT = 128;
     static constexpr int BNT = kRankNT;  // 64
-    static constexpr int KC = KC_;
-    static constexpr int RESIDENT = KC == 16 ? 3 : 2;  // blocks per SM
+    static constexpr int KC = kRankWideKC;
+    static constexpr int RESIDENT = 3;  // blocks per SM
     static constexpr int STAGES = 3;
     static constexpr int CONSUMERS = 128;
     static constexpr int THREADS = CONSUMERS + 32;
@@ -570,11 +560,10 @@ struct WideAcc {
 #pragma unroll
             for (int r = 0; r < 8; ++r) v[r][q] = __ffma2_rn(ad[r], bp[q], v[r][q]);
     }
-    // a full chunk is unrolled whole, so its loads can be scheduled early
     template <int KC>
     __device__ __forceinline__ void chunk(const float *As, const float *Bs, int kcnt, int r0, int c0) {
         if (kcnt == KC) {
-#pragma unroll(KC == 16 ? 8 : KC)
+#pragma unroll 8
             for (int pc = 0; pc < KC; ++pc) step(As, Bs, pc, r0, c0);
         } else {
 #pragma unroll 4
@@ -603,15 +592,6 @@ __device__ __forceinline__ float4 axpby4(float alpha, float4 x, float beta, floa
     return x;
 }
 
-__device__ __forceinline__ void tma_reduce_add_2d_commit(const void *tmap, const void *smem_src, int32_t x,
-                                                         int32_t y) {
-    asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                     reinterpret_cast<uint64_t>(tmap)),
-                 "r"(x), "r"(y), "r"(smem_addr(smem_src))
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
 __device__ __forceinline__ void tma_store_2d_commit(const void *tmap, const void *smem_src, int32_t x,
                                                     int32_t y) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
@@ -622,11 +602,11 @@ __device__ __forceinline__ void tma_store_2d_commit(const void *tmap, const void
 }
 }  // namespace
 
-template <bool TMA_EPI, int KC, int LVC>
-__global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI, KC>::RESIDENT)
+template <bool TMA_EPI, int LVC>
+__global__ void __launch_bounds__(WideCfg<TMA_EPI>::THREADS, WideCfg<TMA_EPI>::RESIDENT)
     rankk_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmC,
                       const RankArgs a, unsigned *status) {
-    using W = WideCfg<TMA_EPI, KC>;
+    using W = WideCfg<TMA_EPI>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *sStage = reinterpret_cast<float *>(smem_raw);
     float *cbuf = sStage + W::STAGES * W::STAGE_ELEMS;
@@ -641,11 +621,6 @@ __global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI
     const int64_t ntiles_total = mtiles * ((a.n + W::BNT - 1) / W::BNT);
     const int nchunks = (int)((a.k + W::KC - 1) / W::KC);
     const bool use_c0 = a.beta != 0.0;
-    // C = C0 + alpha*acc by a TMA reduce-add of the buffer into C (no C0 copy);
-    // FMA-bound shapes only: for k <= 32 the output stream bounds the kernel and the
-    // read-modify-write in L2 streamed slower than the C0 copy (0.43 vs 0.35 ms at
-    // m = n = 16384, k = 32)
-    const bool add_c0 = TMA_EPI && KC == 32 && use_c0 && static_cast<float>(a.beta) == 1.0f;
 
     if (threadIdx.x == 0) {
         prefetch_tmap(&tmA);
@@ -673,10 +648,7 @@ __global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI
             // arrived on cstore) and wait until the store has read the buffer
             auto store_tile = [&](int jj, int32_t x, int32_t y) -> bool {
                 if (!mbar_wait_bounded(cstore, (uint32_t)(jj & 1))) return false;
-                if (add_c0)
-                    tma_reduce_add_2d_commit(&tmC, cbuf, x, y);
-                else
-                    tma_store_2d_commit(&tmC, cbuf, x, y);
+                tma_store_2d_commit(&tmC, cbuf, x, y);
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 return true;
             };
@@ -708,7 +680,7 @@ __global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI
                         }
                         prev_x = (int32_t)i0;
                         prev_y = (int32_t)(tile * W::BNT);
-                        if (use_c0 && !add_c0) {
+                        if (use_c0) {
                             mbar_arrive_expect_tx(cfull, W::C_ELEMS * 4);
                             tma_load_2d(cbuf, &tmC, (int32_t)i0, (int32_t)(tile * W::BNT), cfull, pol_stream);
                         } else {
@@ -777,13 +749,12 @@ __global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI
 #pragma unroll
                 for (int rg = 0; rg < 2; ++rg) {
                     float4 *p = reinterpret_cast<float4 *>(cbuf + cl * W::BMT + r0 + rg * 32);
-                    const bool with_c0 = use_c0 && !add_c0;
                     const float4 x = acc.rows(rg, cc);
-                    if (alpha1 && !with_c0) {
+                    if (alpha1 && !use_c0) {
                         *p = x;
                     } else {
-                        const float4 c0v = with_c0 ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
-                        *p = axpby4(alpha, x, beta, c0v, with_c0);
+                        const float4 c0v = use_c0 ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
+                        *p = axpby4(alpha, x, beta, c0v, use_c0);
                     }
                 }
             }
@@ -847,19 +818,19 @@ __global__ void __launch_bounds__(WideCfg<TMA_EPI, KC>::THREADS, WideCfg<TMA_EPI
     if (!ok && lane == 0) atomicOr(status, kDevErrTimeout);
 }
 
-template <bool TMA_EPI, int KC, int LVC>
+template <bool TMA_EPI, int LVC>
 static cudaError_t launch_rankk_wide_t(const CUtensorMap *tmA, const CUtensorMap *tmC, const RankArgs &a,
                                        unsigned *status, cudaStream_t s) {
-    using W = WideCfg<TMA_EPI, KC>;
+    using W = WideCfg<TMA_EPI>;
     {
         const cudaError_t e =
-            ensure_smem_limit(reinterpret_cast<const void *>(rankk_wide_kernel<TMA_EPI, KC, LVC>), W::SMEM);
+            ensure_smem_limit(reinterpret_cast<const void *>(rankk_wide_kernel<TMA_EPI, LVC>), W::SMEM);
         if (e != cudaSuccess) return e;
     }
     const int64_t tiles = ((a.m + W::BMT - 1) / W::BMT) * ((a.n + W::BNT - 1) / W::BNT);
     const int64_t slots = W::RESIDENT * (int64_t)(a.num_sms > 0 ? a.num_sms : 1);
     const unsigned grid = (unsigned)(tiles < slots ? tiles : slots);
-    rankk_wide_kernel<TMA_EPI, KC, LVC><<<grid, W::THREADS, W::SMEM, s>>>(*tmA, *tmC, a, status);
+    rankk_wide_kernel<TMA_EPI, LVC><<<grid, W::THREADS, W::SMEM, s>>>(*tmA, *tmC, a, status);
     return cudaGetLastError();
 }
 
@@ -910,19 +881,16 @@ static cudaError_t launch_rankk_t(const CUtensorMap *tmA, const CUtensorMap *tmC
     // form of C's accesses: ldc mod (16 bytes / element) for a 16-byte aligned base, else -1
     const int lvc = reinterpret_cast<uintptr_t>(a.C) % 16 == 0 ? (int)((uint64_t)a.ldc % (16 / sizeof(T))) : -1;
     if (tmA) {
-        // FP32 from k = kRankWideMinK on: the 8 x 8-tile kernel (its A tensor map's box is
-        // 128 x rank_wide_kc(k)); C by TMA when its tensor map exists, else in form lvc
-        if (rank_wide(sizeof(T) == 4 ? TSMM_F32 : TSMM_F64, 2, 0, a.k)) {
-            if (rank_wide_kc(a.k) == 16) {
-                if (tmC) return launch_rankk_wide_t<true, 16, 0>(tmA, tmC, a, status, s);
+        // FP32 from k = kRankWideMinK on (its caller sends k >= kRankTcMinK to the tensor cores): the
+        // 8 x 8-tile kernel (its A tensor map's box is 128 x kRankWideKC); C by TMA when its tensor
+        // map exists, else in form lvc
+        if constexpr (std::is_same<T, float>::value) {
+            if (a.k >= kRankWideMinK) {
+                if (tmC) return launch_rankk_wide_t<true, 0>(tmA, tmC, a, status, s);
                 return with_c_form<T>(lvc, [&](auto f) {
-                    return launch_rankk_wide_t<false, 16, decltype(f)::value>(tmA, tmA, a, status, s);
+                    return launch_rankk_wide_t<false, decltype(f)::value>(tmA, tmA, a, status, s);
                 });
             }
-            if (tmC) return launch_rankk_wide_t<true, 32, 0>(tmA, tmC, a, status, s);
-            return with_c_form<T>(lvc, [&](auto f) {
-                return launch_rankk_wide_t<false, 32, decltype(f)::value>(tmA, tmA, a, status, s);
-            });
         }
         // output-bound shapes: one k chunk, C0 prefetched by TMA when it is read
         if (a.k <= Cfg::KC) {
@@ -936,9 +904,10 @@ static cudaError_t launch_rankk_t(const CUtensorMap *tmA, const CUtensorMap *tmC
                 return launch_rankk_tma_t<T, 1, false, false, decltype(f)::value>(tmA, tmA, a, status, s);
             });
         }
-        return with_c_form<T>(lvc, [&](auto f) {
-            return launch_rankk_tma_t<T, 2, false, false, decltype(f)::value>(tmA, tmA, a, status, s);
-        });
+        if constexpr (std::is_same<T, double>::value)
+            return with_c_form<T>(lvc, [&](auto f) {
+                return launch_rankk_tma_t<T, 2, false, false, decltype(f)::value>(tmA, tmA, a, status, s);
+            });
     }
     const int smem = Cfg::KC * (Cfg::BMT + Cfg::BNT) * (int)sizeof(T);
     dim3 grid((unsigned)((a.m + Cfg::BMT - 1) / Cfg::BMT), (unsigned)((a.n + Cfg::BNT - 1) / Cfg::BNT));
