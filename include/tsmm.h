@@ -44,9 +44,9 @@
  *     tensor cores from splits of every entry (errors measured smaller than the
  *     fma chain's): F32 with 16 < n <= 64, or with n > 64 and k > 32, from exact
  *     splits into three BF16 values with all products down to 2^-25 of |a||b|;
- *     F64 with 1 < n <= 64 and
- *     256 <= k <= 2^20 from 56-bit fixed point cut into seven 8-bit digits whose
- *     products are summed exactly.  Inputs such a split cannot carry within the
+ *     F64 with 1 < n <= 64 and 256 <= k <= 2^20, or with n > 64 and k >= 4, from
+ *     55- to 63-bit fixed point cut into 8-bit digits whose products are summed
+ *     exactly.  Inputs such a split cannot carry within the
  *     bound (infinities, NaNs, overflow, extreme or very unevenly scaled
  *     entries) are found by the kernel and computed with fma.
  */

@@ -58,14 +58,14 @@ bool c_tma_ok(const void *C_dev, int64_t ldc, int64_t n, size_t es) {
            (ldc * (int64_t)es) < (1LL << 40) && encoder() != nullptr;
 }
 
-// (Re)encode the plan's cached tensor map of C (box 128-or-bm rows x `cols`)
-// when C's address or stride changed since the last execute.
+// (Re)encode the plan's cached tensor map of C (box rows x cols) when C's address
+// or stride or the kernel (its columns) changed since the last execute.
 tsmm_status encode_tmapc(tsmm_plan_t p, void *C_dev, int64_t m, int64_t n, int64_t ldc, size_t es,
-                         int cols) {
-    if (p->tmapc_ptr == C_dev && p->tmapc_ldc == ldc) return TSMM_OK;
+                         int rows, int cols) {
+    if (p->tmapc_ptr == C_dev && p->tmapc_ldc == ldc && p->tmapc_cols == cols) return TSMM_OK;
     const cuuint64_t gdim[2] = {(cuuint64_t)m, (cuuint64_t)n};
     const cuuint64_t gstride[1] = {(cuuint64_t)(ldc * (int64_t)es)};
-    const cuuint32_t box[2] = {(cuuint32_t)p->bm, (cuuint32_t)cols};
+    const cuuint32_t box[2] = {(cuuint32_t)rows, (cuuint32_t)cols};
     const cuuint32_t estr[2] = {1, 1};
     CUresult r = encoder()(&p->tmapc,
                            p->dtype == TSMM_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -79,6 +79,7 @@ tsmm_status encode_tmapc(tsmm_plan_t p, void *C_dev, int64_t m, int64_t n, int64
     }
     p->tmapc_ptr = C_dev;
     p->tmapc_ldc = ldc;
+    p->tmapc_cols = cols;
     return TSMM_OK;
 }
 
@@ -219,11 +220,17 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
         const size_t off = (size_t)round_up((int64_t)pb->bytes, 256);
         const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
         const bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
-        const bool rtc = rank_tc(dtype, regime, precision, k);
-        cudaError_t e = cudaMalloc(&pb->data, tc     ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float)
-                                              : tc64 ? off + tc64_bytes(k, n)
-                                              : rtc  ? off + rank_tc_bytes(k, pb->ntiles)
-                                                     : pb->bytes);
+        bool rtc = rank_tc(dtype, regime, precision, k), rtc64 = rank_tc64(dtype, regime, precision, k);
+        cudaError_t e = cudaMalloc(&pb->data, tc      ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float)
+                                              : tc64  ? off + tc64_bytes(k, n)
+                                              : rtc   ? off + rank_tc_bytes(k, pb->ntiles)
+                                              : rtc64 ? off + rank_tc64_bytes(k, pb->ntiles)
+                                                      : pb->bytes);
+        if (e != cudaSuccess && (rtc || rtc64)) {  // the panel alone serves the fma kernels
+            cudaGetLastError();
+            rtc = rtc64 = false;
+            e = cudaMalloc(&pb->data, pb->bytes);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             delete pb;
@@ -244,6 +251,11 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
             pb->tc_data = static_cast<char *>(pb->data) + off;
             e = launch_pack_b_rank_tc(k, n, static_cast<const float *>(B_dev), ldb, pb->ntiles, pb->tc_data,
                                       static_cast<cudaStream_t>(stream));
+        }
+        if (e == cudaSuccess && rtc64) {
+            pb->tc_data = static_cast<char *>(pb->data) + off;
+            e = launch_pack_b_rank_tc64(k, n, static_cast<const double *>(B_dev), ldb, pb->ntiles, pb->tc_data,
+                                        static_cast<cudaStream_t>(stream));
         }
         if (e == cudaSuccess && tc64) {
             pb->tc_data = static_cast<char *>(pb->data) + off;
@@ -557,7 +569,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
             // C0 loads and C stores go through TMA when C allows it (any beta)
             const bool tmc = c_tma_ok(C_dev, ldc, n, es);
             if (tmc) {
-                const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, kX3RankSub);
+                const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, p->bm, kX3RankSub);
                 if (st != TSMM_OK) return st;
             }
             // an A that a tensor map cannot describe is moved column by column
@@ -583,6 +595,14 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         ra.alpha = alpha;
         ra.beta = beta;
         ra.num_sms = p->num_sms;
+        if (pb->tc_data && rank_tc64(p->dtype, p->regime, p->precision, k)) {
+            const bool tmc = m < INT_MAX && c_tma_ok(C_dev, ldc, n, es);
+            if (tmc) {
+                const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, kTcRows, kRank64Sub);
+                if (st != TSMM_OK) return st;
+            }
+            return cuda_status(launch_rankk_tc64(tmc ? &p->tmapc : nullptr, ra, p->status, s));
+        }
         // An A that a tensor map cannot describe is small here (k <= 128 columns
         // against an m x n output): it is copied into an aligned scratch buffer
         // from the stream's memory pool (released on the stream after the
@@ -621,19 +641,22 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
                 scratch = nullptr;
             }
         }
-        const bool rtc = tma_a && rank_tc(p->dtype, p->regime, p->precision, k);
+        const bool rtc = tma_a && pb->tc_data && rank_tc(p->dtype, p->regime, p->precision, k);
         // C tiles by TMA (C0 prefetch; C0 and C in the FP32 k > 32 kernel): the
         // same 16-byte rules for C
         const bool tmc = tma_a && c_tma_ok(C_dev, ldc, n, es);
         if (tmc) {
-            const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, rtc ? kRankTcSub : kRankNT);
+            const tsmm_status st = encode_tmapc(p, C_dev, m, n, ldc, es, p->bm, rtc ? kRankTcSub : kRankNT);
             if (st != TSMM_OK) {
                 if (scratch) cudaFreeAsync(scratch, s);
                 return st;
             }
         }
-        const CUtensorMap *ta = tma_a ? (scratch ? &tm_scratch : &p->tmap) : nullptr;
-        const CUtensorMap *tc = tmc ? &p->tmapc : nullptr;
+        // (a B packed without its tensor-core form, for lack of memory, is left to the plain-load kernel: the fma
+        // kernels' tensor copies serve k < kRankTcMinK)
+        const bool plain = !rtc && rank_tc(p->dtype, p->regime, p->precision, k);
+        const CUtensorMap *ta = tma_a && !plain ? (scratch ? &tm_scratch : &p->tmap) : nullptr;
+        const CUtensorMap *tc = tmc && !plain ? &p->tmapc : nullptr;
         const cudaError_t e = rtc ? launch_rankk_tc(ta, tc, ra, p->status, s)
                                   : launch_rankk(p->dtype, ta, tc, ra, p->status, s);
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order

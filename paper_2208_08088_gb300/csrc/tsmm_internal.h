@@ -180,6 +180,7 @@ struct tsmm_plan_s {
     CUtensorMap tmap;
     const void *tmapc_ptr;
     int64_t tmapc_ldc;
+    int tmapc_cols;
     CUtensorMap tmapc;
 };
 
@@ -246,6 +247,18 @@ size_t rank_tc_bytes(int64_t k, int64_t ntiles);
 cudaError_t launch_pack_b_rank_tc(int64_t k, int64_t n, const float *B, int64_t ldb, int64_t ntiles, void *dst, cudaStream_t s);
 cudaError_t launch_rankk_tc(const CUtensorMap *tmA, const CUtensorMap *tmC, const RankArgs &a, unsigned *status,
                             cudaStream_t s);
+// FP64 from k = kRank64TcMinK on (tsmm_rankk_tc64.cu; A read by element, tmC with a box of kTcRows x kRank64Sub): at
+// k = 4, m = n = 16384, beta = 1 the fma kernel took 1.97 ms (FP64 pipe), this one 0.93 at any k <= 32; below 4 the error
+// bound leaves no room for the digits.
+constexpr int kRank64TcMinK = 4;
+constexpr int kRank64Sub = 16;
+inline bool rank_tc64(tsmm_dtype d, int regime, int precision, int64_t k) {
+    return d == TSMM_F64 && regime == 2 && precision == 0 && k >= kRank64TcMinK;
+}
+size_t rank_tc64_bytes(int64_t k, int64_t ntiles);
+cudaError_t launch_pack_b_rank_tc64(int64_t k, int64_t n, const double *B, int64_t ldb, int64_t ntiles, void *dst,
+                                    cudaStream_t s);
+cudaError_t launch_rankk_tc64(const CUtensorMap *tmC, const RankArgs &a, unsigned *status, cudaStream_t s);
 // tmC: tensor map of C (box bm x kRankNT) when C meets the TMA rules, else nullptr.
 cudaError_t launch_rankk(tsmm_dtype dt, const CUtensorMap *tmA, const CUtensorMap *tmC,
                          const RankArgs &a, unsigned *status, cudaStream_t s);

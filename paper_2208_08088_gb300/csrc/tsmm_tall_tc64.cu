@@ -41,28 +41,10 @@ __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int6
     for (int e = threadIdx.x; e < w * (kTc64KB / 2); e += blockDim.x) {
         const int kk = e % (kTc64KB / 2) * 2, j = e / (kTc64KB / 2);
         const int64_t p = (int64_t)blockIdx.x * kTc64KB + kk;
-        uint32_t hi[2], y0[2], y1[2], g = 0u;
-        const int F = j < n ? head->F[j] : kTc64Emin;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const double x = (p + u < k && j < n) ? B[p + u + (int64_t)j * ldb] : 0.0;
-            hi[u] = (uint32_t)__double2hiint(x);
-            const int s = tc64_shift(tc64_abs(hi[u]), F);
-            // one digit more than A: 63 bits below the scale, 0x80 added to the seven low bytes
-            uint64_t m = ((uint64_t)((hi[u] & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x)) << 10;
-            m = s > 63 ? 0ull : m >> (s < 0 ? 0 : s);
-            g |= (uint32_t)(m >> 56) << (8 * u);
-            const uint64_t y = m + 0x0080808080808080ull;
-            y0[u] = (uint32_t)y;
-            y1[u] = (uint32_t)(y >> 32);
-        }
-        const uint32_t sgn = tc64_sign2(hi[0], hi[1]);
-        const uint32_t c = hfma2(sgn, kH1152, 0u);
-        uint32_t d[8];
-        tc64_digits2(y0[0], y0[1], 0x5140, sgn, c, c, d[7], d[6]);
-        tc64_digits2(y0[0], y0[1], 0x7362, sgn, c, c, d[5], d[4]);
-        tc64_digits2(y1[0], y1[1], 0x5140, sgn, c, c, d[3], d[2]);
-        tc64_digits2(y1[0], y1[1], 0x7362, sgn, c, hfma2(sgn, kH1024, 0u), d[1], d[0]);
+        const double *q = B + p + (int64_t)j * ldb;
+        uint32_t d[8];  // A has seven
+        const uint32_t g = tc64_digits8(p < k && j < n ? q[0] : 0.0, p + 1 < k && j < n ? q[1] : 0.0,
+                                        j < n ? head->F[j] : kTc64Emin, d);
         // digit-major rows (digit i, column j) of 16 k: 8-row groups of 256 bytes
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
