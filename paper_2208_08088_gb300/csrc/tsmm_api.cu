@@ -87,6 +87,23 @@ tsmm_status encode_tmapc(tsmm_plan_t p, void *C_dev, int64_t m, int64_t n, int64
 
 namespace tsmm {
 
+int64_t encode_a_rows(CUtensorMap *map, tsmm_dtype dtype, const void *A, int64_t m, int64_t k, int64_t lda) {
+    const int64_t es = (int64_t)dtype_size(dtype), R = 16 / es;
+    const int64_t off = (int64_t)(reinterpret_cast<uintptr_t>(A) % 16) / es;
+    // ends with the last column's last element: no byte behind it is read
+    const int64_t width = off + (R - 1) * lda + m, rows = std::min<int64_t>(k / R, INT_MAX / 2);
+    if (rows < 1 || lda > INT_MAX / 8 || encoder() == nullptr) return 0;
+    const cuuint64_t gdim[2] = {(cuuint64_t)width, (cuuint64_t)rows};
+    const cuuint64_t gstride[1] = {(cuuint64_t)(R * lda * es)};
+    const cuuint32_t box[2] = {(cuuint32_t)(kTcRows + R), (cuuint32_t)kARowsBox};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = encoder()(map, dtype == TSMM_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
+                                 2, const_cast<char *>(static_cast<const char *>(A)) - off * es, gdim, gstride, box, estr,
+                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? rows : 0;
+}
+
 // Costs fitted to sweeps of S on GB300 (m 1000..32768, k 500..32768, every kernel; CUDA graphs of 20 calls).  The sum
 // over the partials is the last block's alone and costs as much per split as one to four stages, which a model of
 // waves and stages alone does not see: m = k = 2048, n = 16: 32 splits 23.8 us, 16 16.0, 8 14.5; m = 1024, n = 64,
@@ -525,6 +542,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
     a.np = p->np;
     a.Bt = pb->tc_data;
     a.bmin = pb->tc_min;
+    a.arows = 0;
 
     const bool tma = aligned(A_dev, 16) && ((lda * (int64_t)es) % 16 == 0) && m < INT_MAX &&
                      k < INT_MAX && (lda * (int64_t)es) < (1LL << 40) && encoder() != nullptr;
@@ -662,8 +680,16 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }
-    if (p->tc && p->dtype == TSMM_F64) return cuda_status(launch_tall_tc64(tma ? &p->tmap : nullptr, a, s));
-    if (p->tc) return cuda_status(launch_tall_tc(tma ? &p->tmap : nullptr, a, s));
+    if (p->tc && !tma) {
+        if (p->tmap_ptr != A_dev || p->tmap_lda != lda) {
+            p->arows = encode_a_rows(&p->tmap, p->dtype, A_dev, m, k, lda);
+            p->tmap_ptr = A_dev;
+            p->tmap_lda = lda;
+        }
+        a.arows = p->arows;
+    }
+    if (p->tc && p->dtype == TSMM_F64) return cuda_status(launch_tall_tc64(p->tmap, !tma, a, s));
+    if (p->tc) return cuda_status(launch_tall_tc(p->tmap, !tma, a, s));
     cudaError_t e = p->dtype == TSMM_F32 ? launch_tall_f32(tma, p->np, &p->tmap, a, s)
                                          : launch_tall_f64(tma, p->np, &p->tmap, a, s);
     return cuda_status(e);

@@ -169,6 +169,7 @@ tsmm_status tsmm::execute_grouped(const tsmm_group_item *items, int count, tsmm_
                 a.np = p->np;
                 a.Bt = it.pb->tc_data;
                 a.bmin = it.pb->tc_min;
+                a.arows = unaligned && lv == kTcForm ? encode_a_rows(&g.tmA, dt, it.A_dev, p->m, p->k, it.lda) : 0;
                 g.item_begin = total;
                 total += n_items;
             }

@@ -178,6 +178,7 @@ struct tsmm_plan_s {
     const void *tmap_ptr;
     int64_t tmap_lda;
     CUtensorMap tmap;
+    int64_t arows;             // tmap is encode_a_rows' with so many rows (tensor-core kernels, unaligned A)
     const void *tmapc_ptr;
     int64_t tmapc_ldc;
     int tmapc_cols;
@@ -200,6 +201,8 @@ struct TallArgs {
     int np;             // row length of Bp, and of the workspace's partial tiles
     const void *Bt;     // tensor-core form of B and its chunks' smallest nonzero magnitudes
     const float *bmin;
+    // tensor-core kernels, A not aligned for a tensor map of its columns: rows of the map of encode_a_rows, 0 without one
+    int64_t arows;
 };
 
 // Launchers (return cudaSuccess or the launch error).  `tma` selects the
@@ -209,9 +212,16 @@ cudaError_t launch_tall_f32(bool tma, int np, const CUtensorMap *tmap, const Tal
 cudaError_t launch_tall_f64(bool tma, int np, const CUtensorMap *tmap, const TallArgs &a,
                             cudaStream_t s);
 
-cudaError_t launch_tall_tc64(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s);
-// The tensor-core kernel; tmap == nullptr: an A that a tensor map cannot describe.
-cudaError_t launch_tall_tc(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s);
+// An A whose column stride is not a multiple of 16 bytes: R = 16 / element size columns together have such a stride, so a
+// map over A's aligned base whose row c spans columns R c .. R c + R - 1 describes it; column R c + q starts in row c at
+// element q * lda + (the base's offset), and a box that begins at the 16-byte boundary below covers eight such columns.
+// Rows of the map: k / R (the columns left are moved one by one); 0 where its coordinates would not fit.
+constexpr int kARowsBox = 8;
+int64_t encode_a_rows(CUtensorMap *map, tsmm_dtype dtype, const void *A, int64_t m, int64_t k, int64_t lda);
+
+// The tensor-core kernels; unaligned: tmap is encode_a_rows' (unused if a.arows == 0).
+cudaError_t launch_tall_tc64(const CUtensorMap &tmap, bool unaligned, const TallArgs &a, cudaStream_t s);
+cudaError_t launch_tall_tc(const CUtensorMap &tmap, bool unaligned, const TallArgs &a, cudaStream_t s);
 
 struct RankArgs {
     int64_t m, n, k, lda, ldc, kp;

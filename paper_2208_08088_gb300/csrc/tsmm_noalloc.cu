@@ -148,6 +148,7 @@ extern "C" tsmm_status tsmm_execute_noalloc(tsmm_dtype dtype, int64_t m, int64_t
     a.kchunk = chunk_stages * kTallBKS;
     a.kp = kp;
     a.slabs = slabs;
+    a.arows = 0;
     a.np = np;
     a.Bt = nullptr;  // the fma kernels (n > 16: their own slab height; the pieces of B would not fit the scratch rule)
     a.bmin = nullptr;

@@ -1,25 +1,20 @@
 // Instantiations and launches of the tensor-core regime (i) kernel, single and grouped.
-#include <cstring>
-
 #include "tsmm_group.cuh"
 #include "tsmm_tall_tc.cuh"
 
 namespace tsmm {
 
 template <int W, bool U>
-static cudaError_t launch_tall_tc_t(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
+static cudaError_t launch_tall_tc_t(const CUtensorMap &tmap, const TallArgs &a, cudaStream_t s) {
     using Cfg = TallTcCfg<W, U>;
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(tall_tc_kernel<W, U>), Cfg::SMEM);
     if (e != cudaSuccess) return e;
-    CUtensorMap none;
-    std::memset(&none, 0, sizeof(none));  // U: never read
     const dim3 grid((unsigned)a.slabs, (unsigned)a.splits);
-    tall_tc_kernel<W, U><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(U ? none : *tmap, a);
+    tall_tc_kernel<W, U><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(tmap, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_tall_tc(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
-    const bool u = tmap == nullptr;
+cudaError_t launch_tall_tc(const CUtensorMap &tmap, bool u, const TallArgs &a, cudaStream_t s) {
     switch (tc_width(a.n)) {
         case 32: return u ? launch_tall_tc_t<32, true>(tmap, a, s) : launch_tall_tc_t<32, false>(tmap, a, s);
         case 48: return u ? launch_tall_tc_t<48, true>(tmap, a, s) : launch_tall_tc_t<48, false>(tmap, a, s);

@@ -27,7 +27,7 @@
 // counters and fixed summation order), 12 warps, two blocks per SM:
 //   warps 0-3   converters: thread = row; FP32 A from shared memory, split, pieces to tensor memory (tcgen05.st)
 //   warps 4-7   promoters: thread = row; chunk sums from tensor memory, added in registers; epilogue
-//   warp 8 (and 11: U)  producers of A: tensor copies, or (U) one bulk copy per column
+//   warp 8      producer of A by tensor copies (U: of every fourth column, encode_a_rows)
 //   warp 9      tensor-memory owner and MMA issuer;  warp 10  producer of packed B chunks
 #pragma once
 #include "tsmm_internal.h"
@@ -42,7 +42,7 @@ template <int W, bool U>
 struct TallTcCfg {
     static constexpr int BM = kTcRows;
     static constexpr int KB = kTcKB;                          // k per chunk (one stage)
-    static constexpr int A_STRIDE = U ? BM + 8 : BM;          // floats per column slot
+    static constexpr int A_STRIDE = U ? BM + 4 : BM;          // floats per column slot (U: column 4 c + q in slot 8 q + c)
     static constexpr int A_BYTES = KB * A_STRIDE * 4;
     static constexpr int PIECE = W * KB * 2;                  // one BF16 piece of a chunk of B
     static constexpr int B_BYTES = 3 * PIECE;
@@ -55,7 +55,6 @@ struct TallTcCfg {
     static constexpr int OFF_BAR = OFF_B + SB * B_BYTES;
     static constexpr int NBAR = 2 * SA + 2 * SB + 8;
     static constexpr int SMEM = OFF_BAR + NBAR * 8 + 32;
-    static constexpr int PRODUCERS = U ? 2 : 1;
     static constexpr int THREADS = 384;
     static constexpr int COL_A = 2 * W;                       // TMEM: 2 accumulators, then 2 x 3 pieces of 16 columns
     static constexpr int TMEM_COLS = 256;
@@ -93,9 +92,9 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     const int64_t i0 = slab * BM;
 
     if (threadIdx.x == 0) {
-        if (!U) prefetch_tmap(tmA);
+        if (!U || a.arows != 0) prefetch_tmap(tmA);
         for (int s = 0; s < SA; ++s) {
-            mbar_init(&afull[s], Cfg::PRODUCERS);
+            mbar_init(&afull[s], 1);
             mbar_init(&aempty[s], 4);
         }
         for (int s = 0; s < SB; ++s) {
@@ -120,7 +119,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
 
     if (warp >= 8) {
         reg_dec<40>();
-        if (warp == 8 || (U && warp == 11)) {
+        if (warp == 8) {
             // ------------------------------------------------ A
             const uint64_t pol = policy_evict_first();
             bool ok = true;
@@ -139,12 +138,14 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
                     }
                 }
             } else {
-                // lane l < 16 of producer w moves column 16 w + l of each stage: one bulk copy of the aligned span
-                // around its rows (column_span_bytes); columns beyond k are zero-filled
+                // Chunks within the map's rows: one tensor copy per q (one bulk copy per column, which the copy engine
+                // takes every 36 cycles an SM, bounded these shapes: m =
+                // 32765, n = 64, k = 32768: 1.00 -> 0.72 ms, m = 141591, n = 39, k = 1607: 231 -> 169 us).
+                // Other chunks: lane = column, one bulk copy of the aligned span around its rows (column_span_bytes);
+                // columns beyond k are zero-filled.
                 const int rows = (int)((a.m - i0 < BM) ? a.m - i0 : BM);
                 const int abase = (int)((reinterpret_cast<uintptr_t>(a.A) / 4) & 3);
                 const int ldv = (int)((uint64_t)a.lda & 3);
-                const int q = (warp == 8 ? 0 : KB / 2) + lane;
                 for (; it < iters; ++it) {
                     const int s = it % SA;
                     if (it >= SA) {
@@ -154,12 +155,21 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
                             break;
                         }
                     }
-                    const int64_t p = k0 + (int64_t)it * KB + q;
-                    float *slot = reinterpret_cast<float *>(smem + s * Cfg::A_BYTES) + q * Cfg::A_STRIDE;
+                    const int64_t pc = k0 + (int64_t)it * KB;
+                    if (pc + KB <= 4 * a.arows) {
+                        if (lane == 0) {
+                            mbar_arrive_expect_tx(&afull[s], Cfg::A_BYTES);
+                            for (int q = 0; q < 4; ++q)
+                                tma_load_2d(smem + s * Cfg::A_BYTES + q * (kARowsBox * Cfg::A_STRIDE * 4), tmA,
+                                            (int32_t)((abase + q * a.lda + i0) & ~(int64_t)3), (int32_t)(pc / 4), &afull[s], pol);
+                        }
+                        continue;
+                    }
+                    const int64_t p = pc + lane;
+                    float *slot = reinterpret_cast<float *>(smem + s * Cfg::A_BYTES) + ((lane & 3) * 8 + lane / 4) * Cfg::A_STRIDE;
                     const int d = (abase + (int)(p & 3) * ldv) & 3;
-                    const bool mine = lane < KB / 2;
-                    const uint32_t bytes = mine && p < a.k ? column_span_bytes<float>(rows, d) : 0u;
-                    if (mine && p >= a.k) {
+                    const uint32_t bytes = p < a.k ? column_span_bytes<float>(rows, d) : 0u;
+                    if (p >= a.k) {
                         for (int r = 0; r < Cfg::A_STRIDE; r += 4)
                             *reinterpret_cast<uint4 *>(slot + r) = make_uint4(0, 0, 0, 0);
                         fence_proxy_async_smem();
@@ -315,7 +325,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
                     const int col = h * 16 + q;
-                    x[q] = U ? src[col * Cfg::A_STRIDE + ((abase + (q & 3) * ldv) & 3)] : src[col * BM];
+                    x[q] = U ? src[((col & 3) * 8 + col / 4) * Cfg::A_STRIDE + ((abase + (q & 3) * ldv) & 3)] : src[col * BM];
                 }
                 uint32_t ph[8], pm[8], pl[8];
 #pragma unroll

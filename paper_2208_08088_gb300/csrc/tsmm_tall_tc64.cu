@@ -1,6 +1,4 @@
 // Packing, instantiations and launch of the FP64 tensor-core regime (i) kernel.
-#include <cstring>
-
 #include "tsmm_group.cuh"
 #include "tsmm_tall_tc64.cuh"
 
@@ -71,19 +69,16 @@ cudaError_t launch_pack_b_tc64(int64_t k, int64_t n, const double *B, int64_t ld
 }
 
 template <int W, bool U>
-static cudaError_t launch_tall_tc64_t(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
+static cudaError_t launch_tall_tc64_t(const CUtensorMap &tmap, const TallArgs &a, cudaStream_t s) {
     using Cfg = TallTc64Cfg<W, U>;
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(tall_tc64_kernel<W, U>), Cfg::SMEM);
     if (e != cudaSuccess) return e;
-    CUtensorMap none;
-    std::memset(&none, 0, sizeof(none));  // U: never read
     const dim3 grid((unsigned)a.slabs, (unsigned)a.splits);
-    tall_tc64_kernel<W, U><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(U ? none : *tmap, a);
+    tall_tc64_kernel<W, U><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(tmap, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_tall_tc64(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
-    const bool u = tmap == nullptr;
+cudaError_t launch_tall_tc64(const CUtensorMap &tmap, bool u, const TallArgs &a, cudaStream_t s) {
     switch (tc64_width(a.n)) {
         case 16: return u ? launch_tall_tc64_t<16, true>(tmap, a, s) : launch_tall_tc64_t<16, false>(tmap, a, s);
         case 32: return u ? launch_tall_tc64_t<32, true>(tmap, a, s) : launch_tall_tc64_t<32, false>(tmap, a, s);

@@ -35,7 +35,8 @@
 //   warps 0-7    converters: thread = row; steps of 16 columns, warps 0-3 the even ones, 4-7 the odd ones (a row's
 //                scale passes from step to step); digits to tensor memory
 //   warps 8-15   promoters: thread = row and half of the columns; guard, exact sums, epilogue
-//   warp 16 (and 19: U)  producers of A;  warp 17 tensor memory and MMAs;  warp 18 producer of the digits of B
+//   warp 16 producer of A (U: tensor copies of every other column, encode_a_rows);  warp 17 tensor memory and MMAs;
+//   warp 18 producer of the digits of B
 #pragma once
 #include "tsmm_internal.h"
 #include "tsmm_finish.cuh"
@@ -49,7 +50,7 @@ struct TallTc64Cfg {
     static constexpr int BM = kTcRows;
     static constexpr int KB = kTc64KB;                        // k per step
     static constexpr int GROUP = 128 / KB;                    // steps per exact group, at most
-    static constexpr int A_STRIDE = U ? BM + 4 : BM;          // doubles per column slot
+    static constexpr int A_STRIDE = U ? BM + 2 : BM;          // doubles per column slot (U: column 2 c + q in slot 8 q + c)
     static constexpr int A_BYTES = KB * A_STRIDE * 8;
     static constexpr int ND = tc64_digits(W);                 // digits of B = orders kept = accumulators
     static constexpr int B_BYTES = ND * W * KB * 2;           // the digits of a step of B, digit-major
@@ -66,7 +67,6 @@ struct TallTc64Cfg {
     static constexpr int OFF_BAR = OFF_F + F_BYTES;
     static constexpr int NBAR = 2 * SA + 2 * SB + 18;
     static constexpr int SMEM = OFF_BAR + NBAR * 8 + 96;
-    static constexpr int PRODUCERS = U ? 2 : 1;
     static constexpr int THREADS = 640;                       // 96 registers each at launch, dealt out again by role:
     static constexpr int CREG = W == 64 ? 72 : 80, PREG = W == 64 ? 144 : W == 48 ? 128 : 112;
     static constexpr int MREG = W == 64 ? 48 : W == 48 ? 64 : 96;
@@ -121,9 +121,9 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     const int iters = (int)((k1 - k0) / KB);
 
     if (threadIdx.x == 0) {
-        if (!U) prefetch_tmap(tmA);
+        if (!U || a.arows != 0) prefetch_tmap(tmA);
         for (int s = 0; s < SA; ++s) {
-            mbar_init(&afull[s], Cfg::PRODUCERS);
+            mbar_init(&afull[s], 1);
             mbar_init(&aempty[s], 4);
         }
         for (int s = 0; s < SB; ++s) {
@@ -160,7 +160,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
 
     if (warp >= 16) {
         reg_dec<Cfg::MREG>();
-        if (warp == 16 || (U && warp == 19)) {
+        if (warp == 16) {
             // ------------------------------------------------ A
             const uint64_t pol = policy_evict_first();
             bool ok = true;
@@ -180,12 +180,13 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                     }
                 }
             } else {
-                // lane l < 8 of producer w moves column 8 w + l of each step: one bulk copy of the aligned span around
-                // its rows (column_span_bytes); columns beyond k are zero-filled
+                // Chunks within the map's rows: one tensor copy per q (tsmm_tall_tc.cuh; m = 32767, n = 4, k = 32768:
+                // 2.14 ms here).
+                // Other chunks: lane = column, one bulk copy of the aligned span around its rows (column_span_bytes);
+                // columns beyond k are zero-filled.
                 const int rows = (int)((a.m - i0 < BM) ? a.m - i0 : BM);
                 const int abase = (int)((reinterpret_cast<uintptr_t>(a.A) / 8) & 1);
                 const int ldv = (int)((uint64_t)a.lda & 1);
-                const int q = (warp == 16 ? 0 : KB / 2) + lane;
                 for (; it < iters; ++it) {
                     const int s = it % SA;
                     if (it == SA && !__all_sync(0xffffffffu, go())) break;
@@ -196,10 +197,20 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                             break;
                         }
                     }
-                    const int64_t p = k0 + (int64_t)it * KB + q;
-                    double *slot = reinterpret_cast<double *>(smem + s * Cfg::A_BYTES) + q * Cfg::A_STRIDE;
+                    const int64_t pc = k0 + (int64_t)it * KB;
+                    if (pc + KB <= 2 * a.arows) {
+                        if (lane == 0) {
+                            mbar_arrive_expect_tx(&afull[s], Cfg::A_BYTES);
+                            for (int q = 0; q < 2; ++q)
+                                tma_load_2d(smem + s * Cfg::A_BYTES + q * (kARowsBox * Cfg::A_STRIDE * 8), tmA,
+                                            (int32_t)((abase + q * a.lda + i0) & ~(int64_t)1), (int32_t)(pc / 2), &afull[s], pol);
+                        }
+                        continue;
+                    }
+                    const int64_t p = pc + lane;
+                    double *slot = reinterpret_cast<double *>(smem + s * Cfg::A_BYTES) + ((lane & 1) * 8 + lane / 2) * Cfg::A_STRIDE;
                     const int d = (abase + (int)(p & 1) * ldv) & 1;
-                    const bool mine = lane < KB / 2;
+                    const bool mine = lane < KB;
                     const uint32_t bytes = mine && p < a.k ? column_span_bytes<double>(rows, d) : 0u;
                     if (mine && p >= a.k) {
                         for (int r = 0; r < Cfg::A_STRIDE; r += 2)
@@ -379,7 +390,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             int mx = 0;
 #pragma unroll
             for (int q = 0; q < KB; ++q) {
-                const double x = U ? src[q * Cfg::A_STRIDE + ((abase + (q & 1) * ldv) & 1)] : src[q * BM];
+                const double x = U ? src[((q & 1) * 8 + q / 2) * Cfg::A_STRIDE + ((abase + (q & 1) * ldv) & 1)] : src[q * BM];
                 hi[q] = (uint32_t)__double2hiint(x);
                 lo[q] = (uint32_t)__double2loint(x);
                 if (U) hi[q] &= vmask;

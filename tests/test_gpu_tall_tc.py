@@ -28,6 +28,18 @@ def test_widths_and_edges(m, n, k, pad):
     assert_parity(C, A, B, C0, 1.5, 0.5, exact=True)
 
 
+@pytest.mark.parametrize("dtype,n,m,k0", [(np.float32, 20, 261, 28), (np.float64, 20, 7000, 256)])
+@pytest.mark.parametrize("dk", [0, 3, 4, 5, 7, 8, 31, 33])  # whole chunks of k by tensor copies, the rest column by column
+@pytest.mark.parametrize("offset,pad", [(0, 1), (0, 2), (1, 0), (2, 3), (3, 1)])
+def test_unaligned_columns(dtype, n, m, k0, dk, offset, pad):
+    """A in NaNs, its columns at every offset from 16 bytes: nothing beside them is used, the last chunk is complete."""
+    k = k0 + dk
+    A, B, C0 = (ti.matrix_np(r, c, s, "integer", dtype) for r, c, s in ((m, k, 21), (k, n, 22), (m, n, 23)))
+    C, pl, _ = run(A, B, C0, 1.0, 1.0, lda=m + pad, a_offset=offset)
+    assert pl.info()["bm"] == 128
+    assert_parity(C, A, B, C0, 1.0, 1.0, exact=True)
+
+
 @pytest.mark.parametrize("lda", [264, 265])  # tensor copies; columns moved one by one
 @pytest.mark.parametrize("n", [24, 40, 64])
 def test_wide_integers_are_exact(n, lda):
