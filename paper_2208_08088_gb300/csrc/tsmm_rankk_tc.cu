@@ -1,13 +1,13 @@
 // Regime (ii), FP32, k > 32, on the tensor cores at FP32 accuracy: C[m x n] = alpha * A[m x k] * B[k x n] + beta * C0.
 //
 // The FMA pipe bounded these shapes (m = n = 16384, k = 64 / 128, beta = 1: 0.567 / 1.063 ms, 0.755 / 0.806 of its
-// peak) where the m x n output stream alone takes 0.32 ms; here 0.355 / 0.369 ms (0.386 under sustained load).  As in regime (i) (tsmm_tall_tc.cuh) every entry is the exact
+// peak) where the m x n output stream alone takes 0.32 ms; here 0.353 / 0.366 ms (0.381 under sustained load).  As in regime (i) (tsmm_tall_tc.cuh) every entry is the exact
 // sum of three BF16 values h + m + l and the six largest products are accumulated in FP32: here the five small ones
 // (l*h, h*l, m*m, m*h, h*m) in one accumulator and h*h in another, added at the end, so that only the k/16 MMAs of h*h
 // round at the size of the sum.  Entries that the split cannot carry (tsmm_tall_tc.cuh) are recomputed per output row
 // of a tile with plain fmas.
 //
-// Persistent blocks, one per SM, walk work items (m-tile of 128 rows, chunk of `rnch` n-tiles of 64 columns), 16 warps:
+// Persistent blocks, one per SM, walk equal shares of the tiles (128 rows x 64 columns), an item per m-tile, 16 warps:
 //   warps 0-3   converters: the item's A tile, FP32 in shared memory -> its pieces in tensor memory (read by every tile)
 //   warp 4      producer: A by tensor copies, packed pieces of B (64 k x 64 columns, 24 KB) through a ring
 //   warp 5      tensor-memory owner and MMA issuer, two pairs of accumulators
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) pack_b_rank_tc_kernel(const float *__rest
 template <int KC>
 __global__ void __launch_bounds__(512, 1)
     rankk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmC, const RankArgs a,
-                    unsigned *status, int c_tma, int rnch) {
+                    unsigned *status, int c_tma) {
     using Cfg = RankTcCfg<KC>;
     constexpr int NB = Cfg::NB, CS = Cfg::CS, BM = Cfg::BM;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -118,10 +118,9 @@ __global__ void __launch_bounds__(512, 1)
 
     const int warp = threadIdx.x / 32;
     const int lane = threadIdx.x % 32;
-    const int64_t mtiles = (a.m + BM - 1) / BM;
     const int64_t ntiles = (a.n + kNT - 1) / kNT;
-    const int64_t nch = (ntiles + rnch - 1) / rnch;
-    const int64_t total = mtiles * nch;
+    const int64_t total = (a.m + BM - 1) / BM * ntiles;
+    const int64_t first = total * blockIdx.x / gridDim.x, last = total * (blockIdx.x + 1) / gridDim.x;
     const bool use_c0 = a.beta != 0.0;
     const int ksteps = (int)((a.k + 15) / 16);
 
@@ -153,14 +152,16 @@ __global__ void __launch_bounds__(512, 1)
     tcf_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
-    // items of this block: f(item's running number, m-tile, first and last n-tile) until it returns false
+    // items of this block, its share of the tiles cut at the m-tiles: f(item's running number, m-tile, first and last
+    // n-tile) until it returns false
     auto items = [&](auto &&f) {
         int j = 0;
-        for (int64_t item = blockIdx.x; item < total; item += gridDim.x, ++j) {
-            int64_t mt, ch;
-            udivmod(item, nch, mt, ch);
-            const int64_t t0 = ch * rnch;
-            if (!f(j, mt, t0, (t0 + rnch < ntiles) ? t0 + rnch : ntiles)) return false;
+        for (int64_t at = first; at < last; ++j) {
+            int64_t mt, t0;
+            udivmod(at, ntiles, mt, t0);
+            const int64_t t1 = t0 + (last - at) < ntiles ? t0 + (last - at) : ntiles;
+            if (!f(j, mt, t0, t1)) return false;
+            at += t1 - t0;
         }
         return true;
     };
@@ -471,18 +472,14 @@ static cudaError_t launch_rank_tc_t(const CUtensorMap *tmA, const CUtensorMap *t
     using Cfg = RankTcCfg<KC>;
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void *>(rankk_tc_kernel<KC>), Cfg::SMEM);
     if (e != cudaSuccess) return e;
-    const int64_t mtiles = (a.m + Cfg::BM - 1) / Cfg::BM, ntiles = (a.n + kNT - 1) / kNT;
+    const int64_t ntiles = (a.n + kNT - 1) / kNT, tiles = (a.m + Cfg::BM - 1) / Cfg::BM * ntiles;
     const int64_t slots = a.num_sms > 0 ? a.num_sms : 1;
-    // n-tiles per item: long items amortise the A tile's load and split, but keep about 4 items a block for balance
-    int64_t rnch = mtiles * ntiles / (4 * slots);
-    rnch = rnch < 1 ? 1 : (rnch > 32 ? 32 : rnch);
-    const int64_t items = mtiles * ((ntiles + rnch - 1) / rnch);
-    const unsigned grid = (unsigned)(items < slots ? items : slots);
+    const unsigned grid = (unsigned)(tiles < slots ? tiles : slots);
     if (grid == 0) return cudaSuccess;
     a.bmin = reinterpret_cast<const uint32_t *>(static_cast<const unsigned char *>(a.Bt) + ntiles * KC * kBCHUNK);
     CUtensorMap none;
     std::memset(&none, 0, sizeof(none));
-    rankk_tc_kernel<KC><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(*tmA, tmC ? *tmC : none, a, status, tmC ? 1 : 0, (int)rnch);
+    rankk_tc_kernel<KC><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(*tmA, tmC ? *tmC : none, a, status, tmC ? 1 : 0);
     return cudaGetLastError();
 }
 
