@@ -312,8 +312,10 @@ def run_reference(args):
 
 # --------------------------------------------------------------------- our arm
 KERNEL_SOURCES = {  # the files that define each kernel family's device code
-    "tall": ["tsmm_tall.cuh", "tsmm_device.cuh"],
-    "rankk": ["tsmm_rankk.cu", "tsmm_device.cuh"],
+    "tall": ["tsmm_tall.cuh", "tsmm_tall_tc.cuh", "tsmm_tall_tc64.cuh", "tsmm_digits64.cuh", "tsmm_finish.cuh", "tsmm_tc.cuh",
+             "tsmm_device.cuh"],
+    "rankk": ["tsmm_rankk.cu", "tsmm_rankk_tc.cu", "tsmm_rankk_tc64.cu", "tsmm_digits64.cuh", "tsmm_tc.cuh",
+              "tsmm_device.cuh"],
 }
 
 
@@ -502,7 +504,8 @@ def time_points(tsmm, torch, pts, tdt, steps, warmup, precision=0, world=1, rank
     es = torch.empty((), dtype=tdt).element_size()
 
     def per_execute(m, pl):
-        copy = precision == 0 and pl.info()["regime"] == 2 and ((m + lda_pad) * es) % 16 != 0
+        copy = (precision == 0 and pl.info()["regime"] == 2 and ((m + lda_pad) * es) % 16 != 0
+                and not (es == 8 and pl.k >= 4))  # the FP64 tensor-core kernel reads A by element
         return pl.launches_per_execute() + (1 if copy else 0)
 
     launches = steps * sum(per_execute(m, plans[(m, n, k)]) for (m, n, k, _) in pts)
@@ -511,10 +514,32 @@ def time_points(tsmm, torch, pts, tdt, steps, warmup, precision=0, world=1, rank
     return points, elapsed_ms, launches, state
 
 
-def rate_points(points, es, hbm_peak, fp_peak_tf):
+def tensor_products(es, n, k):
+    """Tensor-core products per product of the native precision, 0 where the FP pipes compute it (the dispatch rules of
+    tsmm_internal.h; FP64 regime (i) also asks for m * n * k >= 4e7)."""
+    if es == 4:
+        return 6 if n > 16 and (n <= 64 or k > 32) else 0
+    if n > 64:
+        return 36 if k >= 4 else 0
+    return (28 if n > 48 else 35) if n > 1 and k >= 256 else 0
+
+
+def bf16_peak():
+    """Measured dense BF16 / FP16 tensor peak, TFLOP/s."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"])
+    except Exception:
+        return 1900.0
+
+
+def rate_points(points, es, hbm_peak, fp_peak_tf, native=True):
     """Per point: GFLOP/s (Eq. 7), algorithmic GB/s, the roof that binds (the
-    slower of HBM and the FP pipe at their peaks) and the fraction of it."""
+    slower of HBM and the arithmetic pipe at their peaks; native: the tensor
+    cores' over the number of their products where they compute the point) and
+    the fraction of it."""
     out = []
+    fp_pipe_tf, tensor_tf = fp_peak_tf, bf16_peak()
     for p in points:
         m, n, k, beta = p["m"], p["n"], p["k"], p["beta"]
         rows = p["rows"][1] - p["rows"][0]
@@ -522,6 +547,8 @@ def rate_points(points, es, hbm_peak, fp_peak_tf):
         gb = alg_bytes(rows, n, k, beta, es) / 1e9
         gbs = gb / (ms * 1e-3)
         tf = flops(rows, n, k) / (ms * 1e-3) / 1e12
+        products = tensor_products(es, n, k) if native else 0
+        fp_peak_tf = tensor_tf / products if products else fp_pipe_tf
         bound = "hbm" if gb / hbm_peak >= flops(rows, n, k) / (fp_peak_tf * 1e12) else "alu"
         frac = (gbs / hbm_peak) if bound == "hbm" else (tf / fp_peak_tf)
         q = {"m": m, "n": n, "k": k, "beta": beta, "avg_ms": round(ms, 4), "gflops": round(tf * 1e3, 1),
@@ -554,13 +581,8 @@ def run_ours(args):
     peaks = measure_fp_peaks(tsmm)
     hbm_peak, hbm_src = load_peaks()
     if args.precision == "bf16x3":
-        # three BF16 tensor-core products per FP32 product: the measured dense
-        # BF16 peak / 3 (MEASURED_PEAKS.json bf16_tflops)
-        try:
-            with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-                fp_peak_tf = float(json.load(f)["bf16_tflops"]) / 3.0
-        except Exception:
-            fp_peak_tf = 1900.0 / 3.0
+        # three BF16 tensor-core products per FP32 product
+        fp_peak_tf = bf16_peak() / 3.0
         fp_src = "measured dense BF16 peak (MEASURED_PEAKS.json bf16_tflops) / 3 products"
     else:
         key = "fp32" if args.dtype == "f32" else "fp64"
@@ -585,11 +607,15 @@ def run_ours(args):
     else:
         elapsed_ms, value = aggregate_over_ranks(elapsed_ms, step_flops, args.steps, world)
 
-    rated = rate_points(points, es, hbm_peak, fp_peak_tf)
+    rated = rate_points(points, es, hbm_peak, fp_peak_tf, prec == tsmm.PREC_NATIVE)
     dom_i = max(range(len(points)), key=lambda i: points[i]["total_ms"])
     dom = rated[dom_i]
     m, n, k, beta = dom["m"], dom["n"], dom["k"], dom["beta"]
     kernel_key = f"{args.workload}_{args.dtype}_n{n}_k{k}"
+    products = tensor_products(es, n, k) if prec == tsmm.PREC_NATIVE else 0
+    if products:
+        fp_peak_tf = bf16_peak() / products
+        fp_src = f"measured dense BF16 peak (MEASURED_PEAKS.json bf16_tflops) / {products} products"
     if dom["bound"] == "hbm":
         roof = {"bound": "hbm", "achieved": dom["alg_gbs"], "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(dom["alg_gbs"] / hbm_peak, 4),
