@@ -120,10 +120,13 @@ SplitCosts split_costs(tsmm_dtype dt, int np, bool tc, int64_t n) {
         const double stage = 0.28 + 0.0015 * np * np;
         k = {tall_resident_blocks(false, np), stage, stage, tall_block_rows(false, np) * 128.0, 2.5,
              0.5 + 0.1 * np, 0.03 + 0.031 * np, 64.0e6};
-    } else {  // bound by the FP64 pipe above one column
-        const double stage = np == 1 ? 0.66 : 0.54 * np * 2;
-        k = {tall_resident_blocks(true, np), stage, stage, tall_block_rows(true, np) * 256.0, 2.5,
-             0.5 + 0.05 * np, 0.02 + 0.015 * np, 64.0e6};
+    } else if (np == 1) {
+        k = {tall_resident_blocks(true, np), 0.66, 0.66, tall_block_rows(true, np) * 256.0, 2.5, 0.55, 0.035, 64.0e6};
+    } else {
+        // bound by the FP64 pipe, which two blocks share and the sums over the partials take too: m = 1500, n = 64, k = 250:
+        // 4 splits 91 us, 8 104; m = 20000, n = 64, k = 64: 1 split 209 us, 2 215
+        k = {tall_resident_blocks(true, np), 0.54 * np, 1.08 * np, tall_block_rows(true, np) * 256.0, 2.5, 0.19 * np,
+             0.04 * np, 64.0e6, 0.5};
     }
     return k;
 }
@@ -153,7 +156,7 @@ int choose_splits(const SplitCosts &k, int64_t slabs, int64_t kstages, int num_s
             const int64_t waves = full + (rem ? 1 : 0);
             t = (double)waves * ((double)per + 4.0) * stage(resident) + finish;
         } else {
-            t = (double)full * ((double)per * stage(resident) + k.block) +
+            t = (double)full * ((double)per * stage(resident) + k.block + k.share * finish) +
                 (rem ? (double)per * stage(rem) + k.block : 0.0) + finish;
         }
         if (best_t < 0 || t < best_t * (1.0 - 1e-9)) {

@@ -222,4 +222,25 @@ __device__ __forceinline__ Vec<T, N> ld_cg_vec(const T *p) {
     return v;
 }
 
+// s += the partials at src, src + step, ... in order, the loads of up to 8 in flight together.
+template <int G, typename T, int N>
+__device__ __forceinline__ void sum_group(Vec<T, N> &s, const T *&src, int64_t step) {
+    Vec<T, N> t[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) t[u] = ld_cg_vec<T, N>(src + u * step);
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+#pragma unroll
+        for (int r = 0; r < N; ++r) s.v[r] += t[u].v[r];
+    src += G * step;
+}
+template <typename T, int N>
+__device__ __forceinline__ void sum_partials(Vec<T, N> &s, const T *src, int64_t step, int splits) {
+#pragma unroll 1
+    for (int left = splits; left >= 8; left -= 8) sum_group<8>(s, src, step);
+    if (splits & 4) sum_group<4>(s, src, step);
+    if (splits & 2) sum_group<2>(s, src, step);
+    if (splits & 1) sum_group<1>(s, src, step);
+}
+
 }  // namespace tsmm

@@ -10,7 +10,7 @@ namespace tsmm {
 // together, since the sum is otherwise a chain of L2 latencies.
 template <typename T, int THREADS>
 __device__ __forceinline__ void tc_finish(const TallArgs &a, int64_t i0, int t) {
-    constexpr int V = 16 / (int)sizeof(T), PER = kTcRows / V, AHEAD = 8;
+    constexpr int V = 16 / (int)sizeof(T), PER = kTcRows / V;
     const T alpha = static_cast<T>(a.alpha), beta = static_cast<T>(a.beta);
     const int64_t mpad = a.slabs * kTcRows, step = (int64_t)a.np * mpad;
     const T *ws = static_cast<const T *>(a.ws) + i0;
@@ -22,18 +22,7 @@ __device__ __forceinline__ void tc_finish(const TallArgs &a, int64_t i0, int t) 
         Vec<T, V> s;
 #pragma unroll
         for (int u = 0; u < V; ++u) s.v[u] = T(0);
-        for (int sp = 0; sp < a.splits; sp += AHEAD) {
-            Vec<T, V> p[AHEAD];
-#pragma unroll
-            for (int q = 0; q < AHEAD; ++q)
-                if (sp + q < a.splits) p[q] = ld_cg_vec<T, V>(src + (sp + q) * step);
-#pragma unroll
-            for (int q = 0; q < AHEAD; ++q)
-                if (sp + q < a.splits) {
-#pragma unroll
-                    for (int u = 0; u < V; ++u) s.v[u] += p[q].v[u];
-                }
-        }
+        sum_partials(s, src, step, a.splits);
         T *c = static_cast<T *>(a.C) + i0 + r + (int64_t)j * a.ldc;
         if (rows >= V && reinterpret_cast<uintptr_t>(c) % 16 == 0) {
             Vec<T, V> o;

@@ -317,6 +317,7 @@ struct SplitCosts {
     int resident;     // blocks per SM
     double stage, stage2, bytes, block, f0, c;  // stage2: a stage where the SM has another block
     double waves_from;  // bytes of A from which whole waves of stages count at one price (0: never)
+    double share;       // of a slab's sum over the partials, what it takes from the other blocks of a full wave
 };
 SplitCosts split_costs(tsmm_dtype dt, int np, bool tc, int64_t n);
 int choose_splits(const SplitCosts &k, int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits);

@@ -203,19 +203,9 @@ __device__ __forceinline__ void tall_finish(T *red, const TallArgs &a, int64_t s
         // the loads of kAhead splits are in flight together (this block's own partial among them: it was published
         // above), the sums taken in order: one load ahead had made this a chain of L2 latencies, half of a small
         // problem's time (m = k = 2048, n = 16, 38 splits: 40 us a call)
-        constexpr int kAhead = 8;
-        for (int sp = 0; sp < a.splits; sp += kAhead) {
-            Vec<T, R> t[kAhead];
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u)
-                if (sp + u < a.splits) t[u] = ld_cg_vec<T, R>(src + (sp + u) * step);
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u)
-                if (sp + u < a.splits) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) s.v[r] += t[u].v[r];
-                }
-        }
+        // (groups of 8, then the remainder's 4, 2 and 1, under uniform branches: adds of absent splits, though predicated
+        // off, took the FP64 pipe's time; FP64 m = 3008, n = 50, k = 214 on 4 splits: 140 us)
+        sum_partials(s, src, step, a.splits);
         store(q, s);
     }
     if (ctid == 0) a.tickets[slab] = 0u;  // ready for the next launch on this stream
