@@ -261,7 +261,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         } else if (warp == 17) {
             // ------------------------------------------------ MMAs: digit i of A times digit j of B into accumulator i + j.
             // One elected lane walks the loop, unrolled over the ring: its operands stay in uniform registers and it needs
-            // few issue slots in competition with the converters of its scheduler.  28 MMAs of N = W: alone they take 9
+            // few issue slots in competition with the converters of its scheduler.  28 (W = 64) or 35 MMAs of N = W: alone they take 9
             // cycles each at W = 16 and 32 (the tensor pipe's rate) at W = 64, and wider ones no less in sum
             if (elect_one()) {
                 constexpr uint32_t idesc = tc_idesc_f16(BM, W);
