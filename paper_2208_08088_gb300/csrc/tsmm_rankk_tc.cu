@@ -52,8 +52,8 @@ struct RankTcCfg {
 };
 
 __device__ __forceinline__ void store_2d(const void *tmap, const void *src, int32_t x, int32_t y) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];\n\t"
-                 "cp.async.bulk.commit_group;" ::"l"(reinterpret_cast<uint64_t>(tmap)),
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(tmap)),
                  "r"(x), "r"(y), "r"(smem_addr(src))
                  : "memory");
 }
@@ -248,6 +248,9 @@ __global__ void __launch_bounds__(512, 1)
                 if (!mbar_wait_bounded(&c_store[st], (uint32_t)((q / CS) & 1))) return false;
                 if (col0 < a.n)  // boxes wholly past the last column are not issued
                     store_2d(&tmC, cslots + st * (BM * kSUB), (int32_t)(mt * BM), (int32_t)col0);
+                // one group a sub-tile, stored or not: the wait below counts groups, and "all but the newest" has to mean
+                // every sub-tile before this one
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 // with C0 to prefetch into few slots, a slot is freed as early as possible; else the newest store stays in flight
                 if (CS == 4 && use_c0) {
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
