@@ -48,11 +48,12 @@ struct FmaAcc<float, HW> {
 
 // out[0..HW) = columns [c0, c0 + HW) of row `row` of A[:, k0:k1] * B[k0:k1, :], for 256 threads (tid 0..255, named
 // barrier 1) of two column halves x 128 rows.  Packed rows of B arrive by bulk copies into two stages of kFmaRows rows
-// at sb (FP64 with HW = 8: 8 x 128 values more behind them), entries of A a stage ahead in registers; bound by the fma pipe (FP64) or about half of it (FP32).  fbar: two
-// barriers, fresh.  A wait that runs out sets *abort_flag and the status.
+// at sb (FP64 with HW = 8: 8 x 128 values more behind them), entries of A a stage ahead in registers; tot: room for HW x 256
+// values.  Bound by the fma pipe (FP64) or about half of it (FP32).  fbar: two barriers, fresh.  A wait that runs out sets
+// *abort_flag and the status.
 template <typename T, int HW>
 __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t k0, int64_t k1, int c0, T *out, T *sb,
-                                         uint64_t *fbar, unsigned *abort_flag, int tid) {
+                                         T *tot, uint64_t *fbar, unsigned *abort_flag, int tid) {
     constexpr int CH = kFmaRows;
     const int np = a.np;
     const int cols = np - c0;
@@ -91,14 +92,26 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         }
         return true;
     };
+    // Chains of SEG (SEGN) stages, their sums added in `tot`: one chain over a whole item would be several times as long as
+    // the fma kernels', whose blocks split k among warps and more splits (FP64, n = 64, k = 2048, uneven columns: error
+    // 5.5e-16, theirs 3.7e-16, so 2.3e-16).  The totals sit in shared memory because registers for them spill (FP32,
+    // n = 64: 5 times the time).
+    tot += tid;
     // up to 8 columns of FP64 (np <= 8 = HW): the halves share the columns and split each stage's rows, and 16 sums a
     // thread (16 / np rows in turn) cover the FP64 pipe's latency, which one warp per scheduler with 8 sums does not (40 %)
     const int half = tid / 128;
     auto narrow = [&](auto np_tag) {
         constexpr int NPW = decltype(np_tag)::value, SETS = 16 / NPW < CH / 2 ? 16 / NPW : CH / 2;
+        constexpr int SEGN = 8;
         FmaAcc<T, NPW> acc[SETS];
 #pragma unroll
         for (int q = 0; q < SETS; ++q) acc[q].zero();
+        auto sum = [&](int j) {
+            T t = acc[0].get(j);
+#pragma unroll
+            for (int q = 1; q < SETS; ++q) t += acc[q].get(j);
+            return t;
+        };
         T x[CH / 2];
         Ap += (int64_t)(half * (CH / 2)) * a.lda;
 #pragma unroll
@@ -113,15 +126,19 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
                 acc[q % SETS].add(x[q], bs + q * NPW, NPW);
                 x[q] = (in && c + 1 < chunks && q < left) ? __ldg(Ap + (int64_t)q * a.lda) : T(0);
             }
+            if (c % SEGN == SEGN - 1) {
+#pragma unroll
+                for (int j = 0; j < NPW; ++j) tot[j * 256] = c < SEGN ? sum(j) : tot[j * 256] + sum(j);
+#pragma unroll
+                for (int q = 0; q < SETS; ++q) acc[q].zero();
+            }
             if (!stage_next(c)) break;
         }
         T *ex = sb + 2 * CH * 16 + tid % 128;
         T s[NPW];
 #pragma unroll
         for (int j = 0; j < NPW; ++j) {
-            s[j] = acc[0].get(j);
-#pragma unroll
-            for (int q = 1; q < SETS; ++q) s[j] += acc[q].get(j);
+            s[j] = chunks < SEGN ? sum(j) : tot[j * 256] + sum(j);
             if (half == 1) ex[j * 128] = s[j];
         }
         named_barrier(1, 256);
@@ -137,6 +154,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         if (np == 4) return narrow(std::integral_constant<int, 4>{});
         if (np == 8) return narrow(std::integral_constant<int, 8>{});
     }
+    constexpr int SEG = sizeof(T) == 8 ? 1 : 4;
     FmaAcc<T, HW> acc;
     acc.zero();
     T x[CH];
@@ -152,10 +170,15 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
             acc.add(x[q], bs + q * np, cols);
             x[q] = (in && c + 1 < chunks && q < left) ? __ldg(Ap + (int64_t)q * a.lda) : T(0);
         }
+        if (c % SEG == SEG - 1) {
+#pragma unroll
+            for (int j = 0; j < HW; ++j) tot[j * 256] = c < SEG ? acc.get(j) : tot[j * 256] + acc.get(j);
+            acc.zero();
+        }
         if (!stage_next(c)) break;
     }
 #pragma unroll
-    for (int j = 0; j < HW; ++j) out[j] = acc.get(j);
+    for (int j = 0; j < HW; ++j) out[j] = chunks < SEG ? acc.get(j) : tot[j * 256] + acc.get(j);
 }
 
 }  // namespace tsmm

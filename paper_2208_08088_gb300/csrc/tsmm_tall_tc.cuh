@@ -61,8 +61,9 @@ struct TallTcCfg {
     static_assert(SA >= 3, "A ring");
     static_assert(COL_A + 96 <= TMEM_COLS, "tensor memory");
     static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two blocks per SM");
-    static constexpr int OFF_F = BM * (W / 2) * 4;            // fallback, over the A ring: exchange, then rows of B
-    static_assert(OFF_F + 2 * kFmaRows * W * 4 <= SA * A_BYTES, "fallback");
+    static constexpr int OFF_F = BM * (W / 2) * 4;            // fallback, over the A ring: exchange, rows of B, totals
+    static constexpr int OFF_T = OFF_F + 2 * kFmaRows * W * 4;
+    static_assert(OFF_T + 256 * (W / 2) * 4 <= SA * A_BYTES, "fallback");
 };
 
 template <int W, bool U>
@@ -368,8 +369,8 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
         if (stop) return;  // tile not written; the host sees TSMM_ERR_TIMEOUT
         if (redo) {
             float part[HW];
-            fma_item<float, HW>(a, row, k0, k1, 0, part, reinterpret_cast<float *>(smem + Cfg::OFF_F), fbar, abort_flag,
-                                threadIdx.x);
+            fma_item<float, HW>(a, row, k0, k1, 0, part, reinterpret_cast<float *>(smem + Cfg::OFF_F),
+                                reinterpret_cast<float *>(smem + Cfg::OFF_T), fbar, abort_flag, threadIdx.x);
             if (*abort_flag != 0u) return;
 #pragma unroll
             for (int j = 0; j < HW; ++j) ex[j * BM + r] = part[j];
@@ -424,8 +425,8 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
     if (stop) return;
     if (redo) {
-        fma_item<float, HW>(a, row, k0, k1, HW, acc + HW, reinterpret_cast<float *>(smem + Cfg::OFF_F), fbar, abort_flag,
-                            threadIdx.x);
+        fma_item<float, HW>(a, row, k0, k1, HW, acc + HW, reinterpret_cast<float *>(smem + Cfg::OFF_F),
+                            reinterpret_cast<float *>(smem + Cfg::OFF_T), fbar, abort_flag, threadIdx.x);
         if (*abort_flag != 0u) return;
         named_barrier(1, 256);
 #pragma unroll

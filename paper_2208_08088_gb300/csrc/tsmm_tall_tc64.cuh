@@ -81,6 +81,7 @@ struct TallTc64Cfg {
     static_assert(256 * CREG + 256 * PREG + 128 * MREG <= THREADS * 96, "register split");
     static_assert(COL_Y + 24 + COL_SET <= TMEM_COLS, "tensor memory");
     static_assert(kTc64Windows * 64 * W <= F_BYTES, "guard windows");
+    static_assert(256 * (W / 2) * 8 <= SA * A_BYTES, "fallback totals");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
@@ -654,8 +655,14 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     if (stop) return;  // tile not written; the host sees TSMM_ERR_TIMEOUT
     double acc[HW];
     if (redo) {
-        fma_item<double, HW>(a, row, k0, k1, c0, acc, reinterpret_cast<double *>(smem + Cfg::OFF_F), fbar, abort_flag,
-                             threadIdx.x - 256);
+        // its totals lie over the ring of A, where the copies issued ahead of the verdict may still be on their way
+        for (int q = 0; !started && q < SA && q < iters; ++q)
+            if (!mbar_wait_bounded(&afull[q], 0)) {
+                atomicOr(a.status, kDevErrTimeout);
+                atomicOr(abort_flag, 1u);
+            }
+        fma_item<double, HW>(a, row, k0, k1, c0, acc, reinterpret_cast<double *>(smem + Cfg::OFF_F),
+                             reinterpret_cast<double *>(smem), fbar, abort_flag, threadIdx.x - 256);
         if (*abort_flag != 0u) {
             if (a.splits > 1) finish();  // the converters wait there
             return;
