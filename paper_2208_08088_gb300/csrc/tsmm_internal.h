@@ -78,8 +78,10 @@ constexpr int kTc64Emin = 1023 - 400, kTc64Emax = 1023 + 400;  // range of the s
 constexpr int kTc64Windows = 8;
 __host__ __device__ constexpr int tc64_guard(int w) { return w <= 48 ? 1200 : 5120; }
 inline int64_t tc64_width(int64_t n) { return (n + 15) / 16 * 16; }
-// Digits of B, and orders of products, per width: eight where tensor memory holds eight accumulators.
-__host__ __device__ constexpr int tc64_digits(int w) { return w <= 48 ? 8 : 7; }
+// Accumulators per width: one for each of eight orders of products where tensor memory holds eight, else seven.  Rows (of
+// `width` columns) of a packed step of B: its eight digits; or digits 0..5, then digits 0..6 each with the top of the next.
+__host__ __device__ constexpr int tc64_accumulators(int w) { return w <= 48 ? 8 : 7; }
+__host__ __device__ constexpr int tc64_rows(int w) { return w <= 48 ? 8 : 13; }
 // k up to 2^20 keeps the sums' high words below 2^51.
 inline bool tc64_pack(tsmm_dtype d, int regime, int64_t n, int64_t k) {
     return d == TSMM_F64 && regime == 1 && n > 1 && k >= 256 && k <= (1 << 20);
@@ -90,7 +92,7 @@ inline bool tc64_plan(tsmm_dtype d, int regime, int64_t m, int64_t n, int64_t k)
     return tc64_pack(d, regime, n, k) && (double)m * (double)tall_np(n) * (double)k >= 4.0e7;
 }
 // Head of the packed digits of B, in device memory, kTc64Head bytes.  Behind it, for k rounded up to 64: per step of
-// kTc64KB rows tc64_digits digits x width columns, FP16, K-major; then per 64 rows width columns x 64 bytes, the top 7 bits of
+// kTc64KB rows tc64_rows x width columns, FP16, K-major; then per 64 rows width columns x 64 bytes, the top 7 bits of
 // |b| at the column's scale.
 struct TcB64 {
     unsigned bad;               // a nonzero column beyond the scales' range, an infinity or a NaN

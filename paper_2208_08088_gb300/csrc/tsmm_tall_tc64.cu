@@ -34,8 +34,8 @@ __global__ void __launch_bounds__(256) pack_b_tc64_scale_kernel(const double *__
 __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int64_t n, int64_t ldb, int w,
                                    unsigned char *__restrict__ base) {
     const TcB64 *head = reinterpret_cast<const TcB64 *>(base);
-    const int64_t off_guard = kTc64Head + (int64_t)gridDim.x * (tc64_digits(w) * w * kTc64KB * 2);
-    unsigned char *dst = base + kTc64Head + blockIdx.x * (int64_t)(tc64_digits(w) * w * kTc64KB * 2);
+    const int64_t off_guard = kTc64Head + (int64_t)gridDim.x * (tc64_rows(w) * w * kTc64KB * 2);
+    unsigned char *dst = base + kTc64Head + blockIdx.x * (int64_t)(tc64_rows(w) * w * kTc64KB * 2);
     for (int e = threadIdx.x; e < w * (kTc64KB / 2); e += blockDim.x) {
         const int kk = e % (kTc64KB / 2) * 2, j = e / (kTc64KB / 2);
         const int64_t p = (int64_t)blockIdx.x * kTc64KB + kk;
@@ -45,10 +45,12 @@ __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int6
                                         j < n ? head->F[j] : kTc64Emin, d);
         // digit-major rows (digit i, column j) of 16 k: 8-row groups of 256 bytes
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 13; ++i) {
             const int rw = i * w + j;
-            if (i < tc64_digits(w))
-                *reinterpret_cast<uint32_t *>(dst + (rw / 8) * 256 + (kk / 8) * 128 + (rw % 8) * 16 + (kk % 8) * 2) = d[i];
+            if (i >= tc64_rows(w)) break;
+            uint32_t v = d[i & 7];
+            if (tc64_rows(w) == 13 && i >= 6) v = hfma2(d[i - 5], 0x1c001c00u, d[i - 6]);  // d[i-6] + 2^-8 d[i-5], rounded
+            *reinterpret_cast<uint32_t *>(dst + (rw / 8) * 256 + (kk / 8) * 128 + (rw % 8) * 16 + (kk % 8) * 2) = v;
         }
         *reinterpret_cast<uint16_t *>(base + off_guard + (p / 64) * (w * 64) + j * 64 + p % 64) = (uint16_t)g;
     }
@@ -56,7 +58,7 @@ __global__ void pack_b_tc64_kernel(const double *__restrict__ B, int64_t k, int6
 
 size_t tc64_bytes(int64_t k, int64_t n) {
     const int64_t w = tc64_width(n), steps = round_up(k, 64) / kTc64KB;
-    return (size_t)(kTc64Head + steps * tc64_digits((int)w) * w * kTc64KB * 2 + round_up(k, 64) * w);
+    return (size_t)(kTc64Head + steps * tc64_rows((int)w) * w * kTc64KB * 2 + round_up(k, 64) * w);
 }
 
 cudaError_t launch_pack_b_tc64(int64_t k, int64_t n, const double *B, int64_t ldb, void *dst, cudaStream_t s) {

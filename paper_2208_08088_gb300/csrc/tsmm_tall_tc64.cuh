@@ -1,23 +1,32 @@
 // Regime (i), FP64, on the tensor cores at FP64 accuracy: C[m x n] = alpha * A[m x k] * B[k x n] + beta * C0.
 //
 // The FP64 pipe has 4 flop per clock and SM; the FP16 tensor pipe has two thousand times that.  Every row of A (per
-// work item) and every column of B is written in fixed point over a common power of two, X = trunc(|x| 2^(55-E)), and
-// cut into seven signed digits of 8 bits, x = +-sum_i d_i 2^(48-8i) with d in [-128, 128], which FP16 holds
-// exactly.  The product of digit i of A with digit j of B has weight 2^-8(i+j); the 28 products with i + j <= 6 are
-// accumulated on the tensor cores, one FP32 accumulator per order i + j.  Over at most 128 columns of k each of those
-// sums stays below 7 * 128 * 2^14 < 2^24, so it is an exact integer; it is then added to a 96-bit integer in
-// registers.  Nothing is rounded before the end of the item but the truncation of X and the products of order 7 and
-// up: together below 2^-52.7 of 2^E 2^F per term (2^E, 2^F: the powers above the row's and the column's largest
-// entry).  (Splitting a product into exactly accumulated slices: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 2012.)
+// work item) and every column of B is written in fixed point over a common power of two, A as X = trunc(|x| 2^(55-E)) in
+// seven signed digits of 8 bits, x = +-sum_i d_i 2^(48-8i) with d in [-128, 128], B with 63 bits in eight.  FP16 holds a
+// digit exactly.  The product of digit i of A with digit j of B has weight 2^-8(i+j); the products of one order i + j are
+// summed on the tensor cores in an FP32 accumulator of their own.  Over at most 128 columns of k such a sum stays below
+// 7 * 128 * 2^14 < 2^24, so it is an exact integer; it is then added to a 96-bit integer in registers.
+// (Splitting a product into exactly accumulated slices: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 2012.)
+//   W <= 48: the 35 products of orders 0..7, eight accumulators.
+//   W = 64: tensor memory holds seven.  The 28 products of orders 0..6, where order 6 takes, in place of digit j of B,
+//     FP16(d_j + 2^-8 d_(j+1)): its 11 bits bring in order 7 but for 2^-4 of it at no further product (order 7 as products
+//     of its own: 4.09 ms at n = 64 against 3.56; without it, at 3.43 ms, B's rows scaled by 10^U[-3,3] had an
+//     error of 1.3e-15 to 1.7e-15 where the fma kernel's is 3.9e-16 to 5.5e-16).
+// Errors, per term and relative to 2^E 2^F (the powers above the row's and the column's largest entry): 2^-55 of the cut of
+// A, 2^-60 of the orders left out.  Per group of up to 128 columns the sums are rounded to a multiple of 2^-58, and again
+// where the row's scale grows (to a multiple of 2^-54, n = 64 took 3.48 ms but had twice the error on uneven rows).  An
+// entry much smaller than its row's or column's largest is thus held with fewer bits than FP64 has: the error is that of
+// the row's and column's scale, not of each product's own, and the guard below bounds what that may cost.
 //
-// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.45 ms (FP64 pipe 98 % busy before; now 40 TFLOP/s FP64,
-// 2.5 TB/s), n = 32: 55.7 -> 2.56 ms, n = 4: 7.0 -> 1.98 ms (4.3 TB/s); relative error against compensated sums 1.1e-15 to
-// 2.3e-15 -> 1.0e-16 to 1.2e-16, on rows of very different size (n = 8, k = 2048) 2.6e-16 -> 9.7e-17 (without the eighth
-// digit and order 7: 1.4e-15; they cost nothing up to n = 16 and 11 to 20 % above).
+// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.56 ms (FP64 pipe 98 % busy before; now 39 TFLOP/s FP64,
+// 2.4 TB/s), n = 48: 3.20 ms, n = 32: 55.7 -> 2.48 ms, n = 4: 7.0 -> 1.98 ms (4.3 TB/s); relative error against compensated
+// sums, k = 2048 and 8192: uniform entries 2.8e-16 to 5.5e-16 -> 1.2e-16 to 1.9e-16, rows of B scaled by 10^U[-3,3] 3.0e-16
+// to 5.5e-16 -> 1.3e-16 to 1.8e-16, columns of A scaled by 2^U[-2,2] and rows of B by the inverse 2.8e-16 to 5.5e-16 ->
+// 2.0e-16 to 2.4e-16.
 // Bound by issue: a step of 16 columns costs the converters about 2000 warp instructions (HBM alone would leave 710
 // cycles a step, the MMAs take 900 at n = 64, 330 at n <= 16), and at n = 64 by the drains of the accumulators, which
-// tensor memory cannot hold twice there (seven conversions to integers an output had made a drain 4400 cycles; the
-// magic additions below, in one pass: 3.64 -> 3.42 ms).  Two sets of converters, so that one's waits overlap the
+// tensor memory cannot hold twice there (seven conversions to integers an output had made a drain 4400 cycles, and
+// 3.64 ms; two of them are magic additions).  Two sets of converters, so that one's waits overlap the
 // other's work (n = 4: 2.60 -> 2.31 ms); two sets of digits where they fit (n = 4: 2.22 -> 2.03 ms); a single elected MMA
 // lane (n = 64: 3.97 -> 3.64 ms).
 //
@@ -52,9 +61,9 @@ struct TallTc64Cfg {
     static constexpr int GROUP = 128 / KB;                    // steps per exact group, at most
     static constexpr int A_STRIDE = U ? BM + 2 : BM;          // doubles per column slot (U: column 2 c + q in slot 8 q + c)
     static constexpr int A_BYTES = KB * A_STRIDE * 8;
-    static constexpr int ND = tc64_digits(W);                 // digits of B = orders kept = accumulators
-    static constexpr int B_BYTES = ND * W * KB * 2;           // the digits of a step of B, digit-major
-    static constexpr int SA = 8, SB = 4;
+    static constexpr int ND = tc64_accumulators(W);
+    static constexpr int B_BYTES = tc64_rows(W) * W * KB * 2;  // the digits of a step of B, digit-major
+    static constexpr int SA = W == 64 ? 5 : 8, SB = 4;
     static constexpr int OFF_B = SA * A_BYTES;
     static constexpr int OFF_E = OFF_B + SB * B_BYTES;        // row scales of the last ERING steps
     // the guard's digits of B (kTc64Windows windows), later the fallback's rows of B
@@ -71,7 +80,7 @@ struct TallTc64Cfg {
     static constexpr int CREG = W == 64 ? 72 : 80, PREG = W == 64 ? 144 : W == 48 ? 128 : 112;
     static constexpr int MREG = W == 64 ? 48 : W == 48 ? 64 : 96;
     static constexpr int CB = W == 64 ? 4 : 8;                // columns a promoter drains at a time
-    static constexpr int SH = W == 64 ? 0 : 4;                // unit of the sums: 2^-SH of the order-5 products
+    static constexpr int SH = 4;                              // unit of the sums: 2^-SH of the order-5 products
     // tensor memory: ND accumulators of W columns, then the digits of a step of A, 8 columns each: 3-6 (X), 0-2 (Y).
     // DB: two sets of digits, by step parity; else one, whose X and Y parts are refilled in turn
     static constexpr bool DB = W <= 48;
@@ -284,9 +293,10 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                         constexpr int i = decltype(i_tag)::value;
                         static_for<0, Cfg::ND - i>([&](auto j_tag) {
                             constexpr int j = decltype(j_tag)::value;
+                            constexpr int row = Cfg::ND == 7 && i + j == 6 ? 6 + j : j;
                             const uint32_t at = set + (i >= 3 ? Cfg::COL_X + (i - 3) * 8 : Cfg::COL_Y + i * 8);
                             tc_mma_ts2<!(fresh && (i == 3 || (i == 0 && j < 3)))>(acc + (uint32_t)((i + j) * W), at,
-                                                                                  bd + j * (W * 2), bhi, idesc);
+                                                                                  bd + row * (W * 2), bhi, idesc);
                         });
                     });
                 };
@@ -593,6 +603,10 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                     h >>= 32;
                 }
                 if (t > 0) {
+                    // to nearest, ties to even: rows grow at different steps, so an item's sums may be shifted many times
+                    const uint32_t b = ((1u << (t - 1)) - 1u) + (l >> t & 1u);
+                    l += b;
+                    h += l < b ? 1 : 0;
                     l = (l >> t) | ((uint32_t)h << (32 - t));
                     h >>= t;
                 }
@@ -601,12 +615,10 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             }
         }
         // V += 2^SH (2^40 D0 + 2^32 D1 + 2^24 D2 + 2^16 D3 + 2^8 D4 + D5 + 2^-8 D6 + 2^-16 D7).
-        // A conversion to integers takes the XU pipe 8 cycles, so only sums that need their 24 bits go there;
-        // D0 and D1 stay within 2^22 and take a magic addition, and so does at seven orders D5 + 2^-8 D6, rounded to a
-        // multiple of 4 (by 2^-53 of 2^E 2^F at most, once a group).  With all seven converted a drain took 4400 cycles
-        // at W = 64.
+        // (W = 64: without D7, which sits in D6), its lowest part rounded to nearest.  A conversion to integers takes the
+        // XU pipe 8 cycles, so D0 and D1, which stay within 2^22, take a magic addition.
         constexpr int CB = Cfg::CB, SH = Cfg::SH;
-        constexpr uint32_t kM23 = 0x4b400000u, kM25 = 0x4c400000u;  // 1.5 * 2^23, 1.5 * 2^25
+        constexpr uint32_t kM23 = 0x4b400000u;  // 1.5 * 2^23
         const uint32_t acc0 = tlane + (Cfg::DDB ? (uint32_t)(g & 1) * (Cfg::ND * W) : 0u) + c0;
 #pragma unroll
         for (int c = 0; c < HW; c += CB) {
@@ -623,16 +635,19 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                 if constexpr (Cfg::ND == 8) t = fmaf(__uint_as_float(d[7][j]), 0.00390625f, t);
                 t = fmaf(t, 0.00390625f, __uint_as_float(d[5][j]));
                 int64_t L = (int64_t)(uint64_t)vl[c + j];
-                if constexpr (Cfg::ND == 8) L += __float2int_rn(t * 16.f);
-                else L += (int64_t)(int)(__float_as_uint(t + __uint_as_float(kM25)) - kM25) * 4;
+                L += __float2int_rn(t * (float)(1 << SH));
                 L += (int64_t)__float2int_rn(__uint_as_float(d[4][j])) * (1 << (8 + SH));
                 L += (int64_t)__float2int_rn(__uint_as_float(d[3][j])) * (1 << (16 + SH));
                 L += (int64_t)__float2int_rn(__uint_as_float(d[2][j])) * (1 << (24 + SH));
                 vl[c + j] = (uint32_t)L;
                 const uint32_t h = __float_as_uint(__uint_as_float(d[0][j]) + __uint_as_float(kM23)) * 256u +
                                    __float_as_uint(__uint_as_float(d[1][j]) + __uint_as_float(kM23)) - kM23 * 257u;
-                if constexpr (SH == 0) vh[c + j] += (int64_t)((int)h + (int)(L >> 32));
-                else vh[c + j] += (int64_t)(int)h * (1 << SH) + (L >> 32);
+                if constexpr (W == 64) {  // in place: 64-bit temporaries spill here (and in-place costs 1 % below)
+                    vh[c + j] += L >> 32;
+                    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(vh[c + j]) : "r"((int)h), "n"(1 << SH));
+                } else {
+                    vh[c + j] += (int64_t)(int)h * (1 << SH) + (L >> 32);
+                }
             }
         }
         if (slot & 64u) break;
