@@ -21,7 +21,7 @@
 // What the split cannot carry goes another way: a block whose item meets an infinity, a NaN, an overflow (seen as a
 // non-finite sum), or entries so small that a piece of a product could leave FP32's normal range (smallest
 // nonzero |a| times smallest nonzero |b| below 2^-100), recomputes its item with plain fmas (fma_item)
-// before it stores anything, so results follow IEEE fma arithmetic there.
+// before it stores anything, so results follow IEEE fma arithmetic there.  So do products with k < kTcMinK.
 //
 // Block: one work item = one slab of 128 rows x one k range (the split-K scheme of the fma kernel, same workspace,
 // counters and fixed summation order), 12 warps, two blocks per SM:
@@ -109,7 +109,7 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
             mbar_init(&fbar[b], 1);
         }
         *abort_flag = 0u;
-        *unsafe = 0u;
+        *unsafe = a.k < kTcMinK ? 1u : 0u;
         fence_mbar_init();
     }
     if (warp == 9) tc_alloc(tslot, Cfg::TMEM_COLS);
