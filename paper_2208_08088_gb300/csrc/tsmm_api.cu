@@ -547,13 +547,19 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
     a.bmin = pb->tc_min;
     a.arows = 0;
 
+    // A tensor-core plan too short in k for it: the fma kernel on its own slabs (one split: no workspace); the blocks' own
+    // fma path, which grouped launches take, gives the same bits (m = 100000, n = 64, k = 8: 12 us, 50 on the blocks' own)
+    const bool short_k = p->tc && p->dtype == TSMM_F32 && k < kTcMinK;
+    const int bm = short_k ? tall_bm(p->dtype, p->np) : p->bm;
+    if (short_k) a.slabs = (m + bm - 1) / bm;
+
     const bool tma = aligned(A_dev, 16) && ((lda * (int64_t)es) % 16 == 0) && m < INT_MAX &&
                      k < INT_MAX && (lda * (int64_t)es) < (1LL << 40) && encoder() != nullptr;
     if (tma && (p->tmap_ptr != A_dev || p->tmap_lda != lda)) {
         // box: bm rows x 32 columns (the regime (i) stage and the regime (ii) k chunk)
         const cuuint64_t gdim[2] = {(cuuint64_t)m, (cuuint64_t)k};
         const cuuint64_t gstride[1] = {(cuuint64_t)(lda * (int64_t)es)};
-        const cuuint32_t box[2] = {(cuuint32_t)p->bm,
+        const cuuint32_t box[2] = {(cuuint32_t)bm,
                                    (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k, p->tc)};
         const cuuint32_t estr[2] = {1, 1};
         CUresult r = encoder()(&p->tmap,
@@ -683,7 +689,8 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }
-    if (p->tc && !tma) {
+    const bool tc = p->tc && !short_k;
+    if (tc && !tma) {
         if (p->tmap_ptr != A_dev || p->tmap_lda != lda) {
             p->arows = encode_a_rows(&p->tmap, p->dtype, A_dev, m, k, lda);
             p->tmap_ptr = A_dev;
@@ -691,8 +698,8 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         }
         a.arows = p->arows;
     }
-    if (p->tc && p->dtype == TSMM_F64) return cuda_status(launch_tall_tc64(p->tmap, !tma, a, s));
-    if (p->tc) return cuda_status(launch_tall_tc(p->tmap, !tma, a, s));
+    if (tc && p->dtype == TSMM_F64) return cuda_status(launch_tall_tc64(p->tmap, !tma, a, s));
+    if (tc) return cuda_status(launch_tall_tc(p->tmap, !tma, a, s));
     cudaError_t e = p->dtype == TSMM_F32 ? launch_tall_f32(tma, p->np, &p->tmap, a, s)
                                          : launch_tall_f64(tma, p->np, &p->tmap, a, s);
     return cuda_status(e);
