@@ -241,7 +241,7 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
         const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
         const bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
         bool rtc = rank_tc(dtype, regime, precision, k), rtc64 = rank_tc64(dtype, regime, precision, k);
-        cudaError_t e = cudaMalloc(&pb->data, tc      ? off + pieces + (size_t)(pb->kp / kTcKB) * sizeof(float)
+        cudaError_t e = cudaMalloc(&pb->data, tc      ? off + pieces + (size_t)(pb->kp / kTcKB) * 2 * sizeof(float)
                                               : tc64  ? off + tc64_bytes(k, n)
                                               : rtc   ? off + rank_tc_bytes(k, pb->ntiles)
                                               : rtc64 ? off + rank_tc64_bytes(k, pb->ntiles)

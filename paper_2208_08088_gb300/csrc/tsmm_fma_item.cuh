@@ -154,7 +154,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         if (np == 4) return narrow(std::integral_constant<int, 4>{});
         if (np == 8) return narrow(std::integral_constant<int, 8>{});
     }
-    constexpr int SEG = sizeof(T) == 8 ? 1 : 4;
+    constexpr int SEG = sizeof(T) == 8 ? 1 : 8;
     FmaAcc<T, HW> acc;
     acc.zero();
     T x[CH];
@@ -172,7 +172,10 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         }
         if (c % SEG == SEG - 1) {
 #pragma unroll
-            for (int j = 0; j < HW; ++j) tot[j * 256] = c < SEG ? acc.get(j) : tot[j * 256] + acc.get(j);
+            for (int j = 0; j < HW; ++j) {
+                tot[j * 256] = c < SEG ? acc.get(j) : tot[j * 256] + acc.get(j);
+                if (j % 4 == 3) asm volatile("" ::: "memory");  // few of them in registers at a time
+            }
             acc.zero();
         }
         if (!stage_next(c)) break;

@@ -153,7 +153,7 @@ struct tsmm_packed_b_s {
     void *data;      // device storage, kp * w * ntiles elements
     size_t bytes;
     // tensor-core form behind it in the same allocation (nullptr: none): per 32-row chunk of k three BF16 pieces of
-    // tc_width(n) columns, then one float per chunk, the smallest nonzero |B| in it
+    // tc_width(n) columns, then one float per chunk, the smallest nonzero |B| in it, and one more, the largest
     void *tc_data;
     float *tc_min;
 };

@@ -25,24 +25,27 @@ __global__ void pack_b_kernel(const T *__restrict__ B, int64_t k, int64_t n, int
 
 // The regime (i) panel and its tensor-core form (tsmm_tall_tc.cuh) in one pass: block c takes the 32 rows of chunk c
 // (lanes along k, so B is read coalesced), writes the panel rows, the three BF16 pieces of every element at
-// (j/8)*512 + (kk/8)*128 + (j%8)*16 + (kk%8)*2 of its piece, and the chunk's smallest nonzero magnitude.
+// (j/8)*512 + (kk/8)*128 + (j%8)*16 + (kk%8)*2 of its piece, and the chunk's smallest nonzero
+// magnitude (behind all chunks': its largest).
 __global__ void __launch_bounds__(256) pack_b_tc_kernel(const float *__restrict__ B, int64_t k, int64_t n, int64_t ldb,
                                                         float *__restrict__ panel, int np, int w,
                                                         unsigned char *__restrict__ pieces, float *__restrict__ cmin) {
     __shared__ float t[kTcKB][kTallMaxN + 1];
-    __shared__ uint32_t smin;
+    __shared__ uint32_t smin, smax;
     const int64_t p0 = (int64_t)blockIdx.x * kTcKB;
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    if (threadIdx.x == 0) smin = 0xffffffffu;
+    if (threadIdx.x == 0) smin = 0xffffffffu, smax = 0u;
     __syncthreads();
-    uint32_t mn = 0xffffffffu;
+    uint32_t mn = 0xffffffffu, mx = 0u;
     for (int j = warp; j < kTallMaxN; j += 8) {
         const float x = (p0 + lane < k && j < n) ? B[p0 + lane + (int64_t)j * ldb] : 0.f;
         t[lane][j] = x;
         mn = min(mn, __float_as_uint(x) * 2u - 1u);
+        mx = max(mx, __float_as_uint(x) & 0x7fffffffu);
     }
     mn = __reduce_min_sync(0xffffffffu, mn);
-    if (lane == 0) atomicMin(&smin, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) atomicMin(&smin, mn), atomicMax(&smax, mx);
     __syncthreads();
     for (int e = threadIdx.x; e < kTcKB * np; e += 256) panel[p0 * np + e] = t[e / np][e % np];
     unsigned char *dst = pieces + (int64_t)blockIdx.x * (w * kTcKB * 6);
@@ -56,8 +59,10 @@ __global__ void __launch_bounds__(256) pack_b_tc_kernel(const float *__restrict_
         *reinterpret_cast<uint32_t *>(q + piece) = m;
         *reinterpret_cast<uint32_t *>(q + 2 * piece) = l;
     }
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         cmin[blockIdx.x] = smin == 0xffffffffu ? __uint_as_float(0x7f800000u) : __uint_as_float((smin + 1u) >> 1);
+        cmin[gridDim.x + blockIdx.x] = __uint_as_float(smax);
+    }
 }
 
 // C = beta * C0 (beta != 0) or C = 0 (beta == 0, C0 not read).

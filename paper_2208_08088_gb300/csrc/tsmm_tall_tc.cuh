@@ -18,10 +18,15 @@
 // warp stays converged and elects the issuing lane: a loop under `lane == 0` keeps every descriptor in vector registers
 // and took 100 cycles an MMA (0.80 -> 0.70 ms at n = 64).
 //
-// What the split cannot carry goes another way: a block whose item meets an infinity, a NaN, an overflow (seen as a
-// non-finite sum), or entries so small that a piece of a product could leave FP32's normal range (smallest
-// nonzero |a| times smallest nonzero |b| below 2^-100), recomputes its item with plain fmas (fma_item)
-// before it stores anything, so results follow IEEE fma arithmetic there.  So do products with k < kTcMinK.
+// What the split cannot carry goes another way, by plain fmas before anything is stored, so that results follow IEEE fma
+// arithmetic there: rows with an infinity, a NaN or an overflow (seen as a non-finite sum), and rows with a sum so small
+// that what a piece or a piece's product loses below FP32's normal range could show in it.  Where the smallest nonzero
+// |a| of the row times the smallest nonzero |b| of the item is at least 2^-100 nothing is lost; elsewhere the loss is below
+// k 2^-126 (max|a| + max|b| + 8), with max|a| over chunks where B has entries below 2^-108, and a sum 2^26 times that is
+// safe.  (The entries' sizes alone had decided: one entry of 1e-31 in B sent every row of its k range to the fmas; m = k =
+// 8192, n = 64, such an entry in every item: 0.41 -> 0.064 ms, 0.060 without.)  Up to kRedoRows such rows of an item are
+// recomputed on their own (redo_rows; one NaN row a slab: 0.41 -> 0.10 ms), more as a whole item (fma_item; all rows: 0.47
+// ms, the fma kernel 0.15); so are products with k < kTcMinK.
 //
 // Block: one work item = one slab of 128 rows x one k range (the split-K scheme of the fma kernel, same workspace,
 // counters and fixed summation order), 12 warps, two blocks per SM:
@@ -37,6 +42,58 @@
 
 namespace tsmm {
 
+constexpr int kRedoRows = 16;
+
+// Rows i0 + list[0..count) of A[:, k0:k1] * B[k0:k1, :]: the four converter warps take every fourth 32 columns of k each, and
+// leave their sums in out[warp][slot][W]; a lane takes two columns of four rows, A arrives 32 columns of k at a time, one a
+// lane.  Chains of 32 columns, as short as the tensor cores' chunks.  Bound by L2 latency.
+template <int W>
+__device__ __forceinline__ void redo_rows(const TallArgs &a, int64_t i0, int64_t k0, int64_t k1, const unsigned char *list,
+                                          int count, float *out, int warp, int lane) {
+    constexpr int R = 4;
+    const int np = a.np, c = 2 * lane;
+    out += warp * (kRedoRows * W) + c;
+#pragma unroll 1
+    for (int first = 0; first < count; first += R) {
+        const float *A[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            A[q] = static_cast<const float *>(a.A) + i0 + list[first + q < count ? first + q : first];
+        float2 sum[R];
+        float x[R], y[R];
+        auto load = [&](int64_t p) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) y[q] = p < a.k ? __ldg(A[q] + p * a.lda) : 0.f;
+        };
+#pragma unroll
+        for (int q = 0; q < R; ++q) sum[q] = make_float2(0.f, 0.f);
+        load(k0 + 32 * warp + lane);
+#pragma unroll 1
+        for (int64_t p = k0 + 32 * warp; p < k1; p += 128) {
+            const float *B = static_cast<const float *>(a.Bp) + p * np + (c < np ? c : 0);
+#pragma unroll
+            for (int q = 0; q < R; ++q) x[q] = y[q];
+            load(p + 128 + lane);
+            float2 s[R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) s[q] = make_float2(0.f, 0.f);
+#pragma unroll 16
+            for (int u = 0; u < 32; ++u) {
+                const float2 b = __ldg(reinterpret_cast<const float2 *>(B + u * np));
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const float v = __shfl_sync(0xffffffffu, x[q], u);
+                    s[q] = __ffma2_rn(make_float2(v, v), b, s[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < R; ++q) sum[q] = __fadd2_rn(sum[q], s[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            if (first + q < count && c < W) *reinterpret_cast<float2 *>(out + (first + q) * W) = sum[q];
+    }
+}
 
 template <int W, bool U>
 struct TallTcCfg {
@@ -54,7 +111,8 @@ struct TallTcCfg {
     static constexpr int OFF_B = SA * A_BYTES;
     static constexpr int OFF_BAR = OFF_B + SB * B_BYTES;
     static constexpr int NBAR = 2 * SA + 2 * SB + 8;
-    static constexpr int SMEM = OFF_BAR + NBAR * 8 + 32;
+    static constexpr int OFF_THR = OFF_BAR + NBAR * 8 + 48;   // rows' least safe sums, then the list of unsafe rows
+    static constexpr int SMEM = OFF_THR + BM * 4 + kRedoRows;
     static constexpr int THREADS = 384;
     static constexpr int COL_A = 2 * W;                       // TMEM: 2 accumulators, then 2 x 3 pieces of 16 columns
     static constexpr int TMEM_COLS = 256;
@@ -63,7 +121,7 @@ struct TallTcCfg {
     static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two blocks per SM");
     static constexpr int OFF_F = BM * (W / 2) * 4;            // fallback, over the A ring: exchange, rows of B, totals
     static constexpr int OFF_T = OFF_F + 2 * kFmaRows * W * 4;
-    static_assert(OFF_T + 256 * (W / 2) * 4 <= SA * A_BYTES, "fallback");
+    static_assert(OFF_T + 256 * (W / 2) * 4 <= SA * A_BYTES && 4 * kRedoRows * W * 4 <= OFF_F, "fallback");
 };
 
 template <int W, bool U>
@@ -83,7 +141,10 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
     unsigned *tslot = reinterpret_cast<unsigned *>(bar + Cfg::NBAR);
     unsigned *flag = tslot + 1;
     unsigned *abort_flag = tslot + 2;
-    unsigned *unsafe = tslot + 3;
+    unsigned *unsafe = tslot + 3;      // rows to recompute
+    unsigned *doubt = tslot + 4;       // some row has entries small enough to ask its sums
+    float *thr = reinterpret_cast<float *>(smem + Cfg::OFF_THR);
+    unsigned char *list = smem + Cfg::OFF_THR + BM * 4;
 
     const int warp = threadIdx.x / 32;
     const int lane = threadIdx.x % 32;
@@ -109,7 +170,8 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
             mbar_init(&fbar[b], 1);
         }
         *abort_flag = 0u;
-        *unsafe = a.k < kTcMinK ? 1u : 0u;
+        *unsafe = a.k < kTcMinK ? kRedoRows + 1u : 0u;
+        *doubt = 0u;
         fence_mbar_init();
     }
     if (warp == 9) tc_alloc(tslot, Cfg::TMEM_COLS);
@@ -362,18 +424,44 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
         }
         const float amn = amin == 0xffffffffu ? __uint_as_float(0x7f800000u) : __uint_as_float((amin + 1u) >> 1);
         constexpr float kTiny = 7.8886091e-31f;  // 2^-100
-        if (row < a.m && !(amn >= kTiny && bmin >= kTiny && amn * bmin >= kTiny)) *unsafe = 1u;
-        // every converter and promoter warp gets here (bounded waits); the flags are read between two barriers
+        float least = 0.f;
+        const bool small = row < a.m && !(amn >= kTiny && bmin >= kTiny && amn * bmin >= kTiny);
+        if (__any_sync(0xffffffffu, small)) {
+            // largest |b|, and |a| in the chunks of k where pieces of B may be lost (tracked in the loop above, 2 % of it)
+            const float *bm = a.bmin + k0 / KB;
+            float ax = 0.f, bx = 0.f;
+            for (int c = 0; c < iters; ++c) {
+                bx = fmaxf(bx, __ldg(bm + a.kp / KB + c));
+                if (__ldg(bm + c) < 3.0814879e-33f) {  // 2^-108
+                    const float *Ar = static_cast<const float *>(a.A) + (row < a.m ? row : 0);
+                    const int64_t p = k0 + (int64_t)c * KB;
+                    float y[KB];
+#pragma unroll
+                    for (int q = 0; q < KB; ++q) y[q] = p + q < a.k ? __ldg(Ar + (p + q) * a.lda) : 0.f;
+#pragma unroll
+                    for (int q = 0; q < KB; ++q) ax = fmaxf(ax, fabsf(y[q]));
+                }
+            }
+            if (small) least = (float)(k1 - k0) * 1.5777218e-30f * (ax + bx + 4.f);  // 2^-99
+            *doubt = 1u;
+        }
+        thr[r] = least;
+        // every converter and promoter warp gets here (bounded waits); the flags are read between barriers
         named_barrier(1, 256);
-        const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
+        named_barrier(1, 256);
+        const bool stop = *abort_flag != 0u;
+        const unsigned redo = *unsafe;
         if (stop) return;  // tile not written; the host sees TSMM_ERR_TIMEOUT
-        if (redo) {
+        if (redo > kRedoRows) {
             float part[HW];
             fma_item<float, HW>(a, row, k0, k1, 0, part, reinterpret_cast<float *>(smem + Cfg::OFF_F),
                                 reinterpret_cast<float *>(smem + Cfg::OFF_T), fbar, abort_flag, threadIdx.x);
             if (*abort_flag != 0u) return;
 #pragma unroll
             for (int j = 0; j < HW; ++j) ex[j * BM + r] = part[j];
+            named_barrier(1, 256);
+        } else if (redo != 0u) {
+            redo_rows<W>(a, i0, k0, k1, list, (int)redo, ex, warp, lane);
             named_barrier(1, 256);
         }
         if (a.splits > 1) finish();
@@ -420,17 +508,38 @@ __device__ __forceinline__ void tall_tc_block(const CUtensorMap *tmA, const Tall
         float z = 0.f;  // 0 unless a sum is infinite or NaN
 #pragma unroll
         for (int j = 0; j < W; ++j) z = fmaf(acc[j], 0.f, z);
-        if (row < a.m && z != 0.f) *unsafe = 1u;
     named_barrier(1, 256);
-    const bool stop = *abort_flag != 0u, redo = *unsafe != 0u;
+    bool bad = z != 0.f;
+    if (*doubt != 0u) {
+        const float least = thr[r];
+#pragma unroll
+        for (int j = 0; j < W; ++j) bad |= j < n && fabsf(acc[j]) < least;
+    }
+    unsigned slot = kRedoRows;
+    if (bad && row < a.m) {
+        slot = atomicAdd(unsafe, 1u);
+        if (slot < kRedoRows) list[slot] = (unsigned char)r;
+    }
+    named_barrier(1, 256);
+    const bool stop = *abort_flag != 0u;
+    const unsigned redo = *unsafe;
     if (stop) return;
-    if (redo) {
+    if (redo > kRedoRows) {
         fma_item<float, HW>(a, row, k0, k1, HW, acc + HW, reinterpret_cast<float *>(smem + Cfg::OFF_F),
                             reinterpret_cast<float *>(smem + Cfg::OFF_T), fbar, abort_flag, threadIdx.x);
         if (*abort_flag != 0u) return;
         named_barrier(1, 256);
 #pragma unroll
         for (int j = 0; j < HW; ++j) acc[j] = ex[j * BM + r];
+    } else if (redo != 0u) {
+        named_barrier(1, 256);
+        if (slot < kRedoRows) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                const float *e = ex + slot * W + j;
+                acc[j] = e[0] + e[kRedoRows * W] + e[2 * kRedoRows * W] + e[3 * kRedoRows * W];
+            }
+        }
     }
     if (a.splits == 1) {
 #pragma unroll
