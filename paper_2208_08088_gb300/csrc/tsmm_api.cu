@@ -588,7 +588,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
             ra.A = A_dev;
             ra.Bp = pb->data;
             ra.Bt = nullptr;
-            ra.bmin = nullptr;
+            ra.brange = nullptr;
             ra.C = C_dev;
             ra.alpha = alpha;
             ra.beta = beta;
@@ -617,7 +617,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         ra.A = A_dev;
         ra.Bp = pb->data;
         ra.Bt = pb->tc_data;
-        ra.bmin = nullptr;
+        ra.brange = nullptr;
         ra.C = C_dev;
         ra.alpha = alpha;
         ra.beta = beta;

@@ -236,8 +236,8 @@ struct RankArgs {
     void *C;
     double alpha, beta;
     int num_sms;     // persistent grid size = resident blocks x SMs
-    const void *Bt;         // tensor-core form of B, and the smallest magnitudes in its chunks
-    const uint32_t *bmin;
+    const void *Bt;         // tensor-core form of B, and the smallest and largest magnitudes in its chunks
+    const uint2 *brange;
 };
 // tmA: tensor map of A (box bm x 32) or nullptr for the plain-load kernel;
 // The FP32 regime (ii) kernel for k in kRankWideMinK..32 streams k in chunks of kRankWideKC, so its A

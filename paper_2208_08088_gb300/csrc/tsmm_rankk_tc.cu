@@ -4,8 +4,8 @@
 // peak) where the m x n output stream alone takes 0.32 ms; here 0.353 / 0.366 ms (0.381 under sustained load).  As in regime (i) (tsmm_tall_tc.cuh) every entry is the exact
 // sum of three BF16 values h + m + l and the six largest products are accumulated in FP32: here the five small ones
 // (l*h, h*l, m*m, m*h, h*m) in one accumulator and h*h in another, added at the end, so that only the k/16 MMAs of h*h
-// round at the size of the sum.  Entries that the split cannot carry (tsmm_tall_tc.cuh) are recomputed per output row
-// of a tile with plain fmas.
+// round at the size of the sum.  What the split cannot carry (tsmm_tall_tc.cuh: non-finite sums, and sums too small for
+// the entries that make them up) is recomputed per output row of a tile with plain fmas.
 //
 // Persistent blocks, one per SM, walk equal shares of the tiles (128 rows x 64 columns), an item per m-tile, 16 warps:
 //   warps 0-3   converters: the item's A tile, FP32 in shared memory -> its pieces in tensor memory (read by every tile)
@@ -36,8 +36,8 @@ struct RankTcCfg {
     static constexpr int NB = 4;                       // B chunk buffers
     static constexpr int CS = KC == 1 ? 6 : 4;         // C slots; even, so that a slot always serves the same half
     static constexpr int SLOT = BM * kSUB * 4;
-    static constexpr int OFF_E = 512;                  // smallest exponents of A's rows, 4 items x 128 bytes
-    static constexpr int OFF_A = 1024;
+    static constexpr int OFF_E = 512;                  // smallest and largest exponents of A's rows, 4 items x 128 x 2 bytes
+    static constexpr int OFF_A = OFF_E + 4 * BM * 2;
     static constexpr int OFF_B = OFF_A + A_BYTES;
     static constexpr int OFF_C = OFF_B + NB * kBCHUNK;
     static constexpr int SMEM = OFF_C + CS * SLOT;
@@ -62,24 +62,71 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity) {
     return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity));
 }
 
+// v[jj] = row `lane` of A times column jj of B (packed, kNT to a row) by plain fmas, for the lanes in `rows`.  Not inlined: its
+// registers would spill the epilogue's.
+__noinline__ __device__ void redo_rows(const float *A, int64_t lda, int64_t k, const float *Bp, unsigned rows, float *v) {
+    const int lane = threadIdx.x % 32;
+    if (__popc(rows) <= 8) {
+        // few rows: one by one, lane = column, A 32 columns of k at a time
+        for (; rows != 0u; rows &= rows - 1u) {
+            const int src = __ffs((int)rows) - 1;
+            float s = 0.f;
+#pragma unroll 1
+            for (int64_t p = 0; p < k; p += 32) {
+                const float x = p + lane < k ? __ldg(A + src + (p + lane) * lda) : 0.f;
+                const int left = (int)min((int64_t)32, k - p);
+#pragma unroll 16
+                for (int u = 0; u < 32; ++u) {
+                    const float b = u < left ? __ldg(Bp + (p + u) * kNT + lane) : 0.f;
+                    s = fmaf(__shfl_sync(0xffffffffu, x, u), b, s);
+                }
+            }
+            for (int jj = 0; jj < 32; ++jj) {
+                const float o = __shfl_sync(0xffffffffu, s, jj);
+                if (lane == src) v[jj] = o;
+            }
+        }
+        return;
+    }
+    const bool mine = rows >> lane & 1u;
+    float2 s[16];
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) s[jj] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int64_t p = 0; p < k; ++p) {
+        const float x = mine ? __ldg(A + lane + p * lda) : 0.f;
+        const float2 x2 = make_float2(x, x);
+#pragma unroll
+        for (int jj = 0; jj < 16; jj += 2) {
+            const float4 b = __ldg(reinterpret_cast<const float4 *>(Bp + p * kNT + 2 * jj));
+            s[jj] = __ffma2_rn(x2, make_float2(b.x, b.y), s[jj]);
+            s[jj + 1] = __ffma2_rn(x2, make_float2(b.z, b.w), s[jj + 1]);
+        }
+    }
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj)
+        if (mine) v[jj] = jj & 1 ? s[jj / 2].y : s[jj / 2].x;
+}
+
 }  // namespace
 
 // Pieces of B: block (tile, chunk), per column j and k kk of a piece at (j/8)*1024 + (kk/8)*128 + (j%8)*16 + (kk%8)*2,
-// and the smallest 2|b| - 1 (bits) over the chunk's nonzero entries.
+// and the smallest and the largest 2|b| - 1 (bits) over the chunk's nonzero entries (0 for the largest of none).
 __global__ void __launch_bounds__(256) pack_b_rank_tc_kernel(const float *__restrict__ B, int64_t k, int64_t n, int64_t ldb,
-                                                             unsigned char *__restrict__ dst, uint32_t *__restrict__ bmin) {
-    __shared__ uint32_t smin;
-    if (threadIdx.x == 0) smin = 0xffffffffu;
+                                                             unsigned char *__restrict__ dst, uint2 *__restrict__ brange) {
+    __shared__ uint32_t smin, smax;
+    if (threadIdx.x == 0) smin = 0xffffffffu, smax = 0u;
     __syncthreads();
     const int64_t at = (int64_t)blockIdx.x * gridDim.y + blockIdx.y;
     unsigned char *chunk = dst + at * kBCHUNK;
-    uint32_t mn = 0xffffffffu;
+    uint32_t mn = 0xffffffffu, mx = 0u;
     for (int e = threadIdx.x; e < kNT * kKB / 2; e += 256) {
         const int j = e / (kKB / 2), kk = e % (kKB / 2) * 2;
         const int64_t col = (int64_t)blockIdx.x * kNT + j, p = (int64_t)blockIdx.y * kKB + kk;
         const float x0 = (col < n && p < k) ? B[p + col * ldb] : 0.f;
         const float x1 = (col < n && p + 1 < k) ? B[p + 1 + col * ldb] : 0.f;
         mn = min(mn, min(__float_as_uint(x0) * 2u - 1u, __float_as_uint(x1) * 2u - 1u));
+        mx = max(mx, max(__float_as_uint(x0) * 2u, __float_as_uint(x1) * 2u));
         uint32_t h, m, l;
         split3_bf16x2(x0, x1, h, m, l);
         unsigned char *q = chunk + (j / 8) * 1024 + (kk / 8) * 128 + (j % 8) * 16 + (kk % 8) * 2;
@@ -88,9 +135,10 @@ __global__ void __launch_bounds__(256) pack_b_rank_tc_kernel(const float *__rest
         *reinterpret_cast<uint32_t *>(q + 2 * kPIECE) = l;
     }
     mn = __reduce_min_sync(0xffffffffu, mn);
-    if (threadIdx.x % 32 == 0) atomicMin(&smin, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (threadIdx.x % 32 == 0) atomicMin(&smin, mn), atomicMax(&smax, mx);
     __syncthreads();
-    if (threadIdx.x == 0) bmin[at] = smin;
+    if (threadIdx.x == 0) brange[at] = make_uint2(smin, smax == 0u ? 0u : smax - 1u);
 }
 
 template <int KC>
@@ -113,7 +161,7 @@ __global__ void __launch_bounds__(512, 1)
     uint64_t *c_store = c_full + CS;    // [CS] results written to it
     uint64_t *c_empty = c_store + CS;   // [CS] slot free
     unsigned *tslot = reinterpret_cast<unsigned *>(bar + Cfg::NBAR);
-    unsigned char *rowexp = smem + Cfg::OFF_E;  // [4][BM]
+    uchar2 *rowexp = reinterpret_cast<uchar2 *>(smem + Cfg::OFF_E);  // [4][BM]
     float *cslots = reinterpret_cast<float *>(smem + Cfg::OFF_C);
 
     const int warp = threadIdx.x / 32;
@@ -340,7 +388,7 @@ __global__ void __launch_bounds__(512, 1)
             tcf_after();
             const float *src = reinterpret_cast<const float *>(smem + Cfg::OFF_A) + r;
             const uint32_t at = tlane + Cfg::COL_A + (Cfg::A_BUFS == 2 ? j & 1 : 0) * Cfg::A_COLS;
-            uint32_t mn = 0xffffffffu;
+            uint32_t mn = 0xffffffffu, mx = 0u;
 #pragma unroll 1
             for (int ks = 0; ks < ksteps; ++ks) {
                 float x[16];
@@ -351,6 +399,7 @@ __global__ void __launch_bounds__(512, 1)
                 for (int q = 0; q < 8; ++q) {
                     mn = min(mn, __float_as_uint(x[2 * q]) * 2u - 1u);
                     mn = min(mn, __float_as_uint(x[2 * q + 1]) * 2u - 1u);
+                    mx = max(mx, max(__float_as_uint(x[2 * q]) * 2u, __float_as_uint(x[2 * q + 1]) * 2u));
                     split3_bf16x2(x[2 * q], x[2 * q + 1], ph[q], pm[q], pl[q]);
                 }
                 const uint32_t t = at + (ks / 4) * 96 + (ks % 4) * 8;
@@ -358,8 +407,9 @@ __global__ void __launch_bounds__(512, 1)
                 tc_st8(t + 32, pm);
                 tc_st8(t + 64, pl);
             }
-            // exponent field of the smallest nonzero entry (255: none)
-            rowexp[(j & 3) * BM + r] = mn == 0xffffffffu ? 255 : (unsigned char)((mn + 1u) >> 24);
+            // exponent fields of the smallest nonzero entry (255: none) and of the largest
+            rowexp[(j & 3) * BM + r] = make_uchar2(mn == 0xffffffffu ? 255 : (unsigned char)((mn + 1u) >> 24),
+                                                   (unsigned char)(mx >> 24));
             release_reads_to_async_copy();
             tc_wait_st();
             tcf_before();
@@ -385,14 +435,18 @@ __global__ void __launch_bounds__(512, 1)
         const int64_t i = mt * BM + r;
         for (int64_t t = t0; t < t1; ++t, ++g, q += 2) {
             const int tb = g & 1;
-            uint32_t bm = __ldg(a.bmin + t * KC);
-            if (KC == 2) bm = min(bm, __ldg(a.bmin + t * KC + 1));
+            uint2 br = __ldg(a.brange + t * KC);
+            if (KC == 2) {
+                const uint2 b1 = __ldg(a.brange + t * KC + 1);
+                br.x = min(br.x, b1.x);
+                br.y = max(br.y, b1.y);
+            }
             if (!warp_wait(&tfull[tb], (uint32_t)((g >> 1) & 1))) return false;
             tcf_after();
             uint32_t vh[32], vl[32];
             tc_ld32(tlane + tb * (2 * kNT) + half * 32, vh);
             tc_ld32(tlane + tb * (2 * kNT) + kNT + half * 32, vl);
-            const int ea = rowexp[(j & 3) * BM + r];
+            const uchar2 ea = rowexp[(j & 3) * BM + r];
             tcf_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[tb]);
@@ -403,23 +457,30 @@ __global__ void __launch_bounds__(512, 1)
                 v[jj] = __uint_as_float(vh[jj]) + __uint_as_float(vl[jj]);
                 z = fmaf(v[jj], 0.f, z);
             }
-            const int eb = bm == 0xffffffffu ? 255 : (int)((bm + 1u) >> 24);
-            const bool redo = i < a.m && (z != 0.f || ea < 27 || eb < 27 || ea + eb < 2 * 127 - 100);
-            if (__any_sync(0xffffffffu, redo)) {
-                // plain fmas from the packed panel, for the rows that need them
-                const float *Bp = static_cast<const float *>(a.Bp) + t * a.kp * kNT + half * 32;
-                const float *Ap = static_cast<const float *>(a.A) + (i < a.m ? i : 0);
-                float s[32];
+            const int eb = br.x == 0xffffffffu ? 255 : (int)((br.x + 1u) >> 24);
+            const bool small = ea.x < 27 || eb < 27 || ea.x + eb < 2 * 127 - 100;
+            if (__any_sync(0xffffffffu, i < a.m && (z != 0.f || small))) {
+                bool redo = z != 0.f;
+                // Entries so small that a piece or a product may have left FP32's normal range: the loss is below
+                // k 2^-126 (max|a| + max|b| + 8), k <= 128, and a sum is safe from 2^26 times that on (2^(e - 217) here).
+                if (small) {
+                    const int e = max(130, max((int)ea.y, (int)((br.y + 1u) >> 24)));
+                    const float least = __uint_as_float((uint32_t)min(255, e - 90) << 23);
+                    const int cols = (int)min((int64_t)32, a.n - (t * kNT + half * 32));
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj) s[jj] = 0.f;
-                for (int64_t p = 0; p < a.k; ++p) {
-                    const float x = __ldg(Ap + p * a.lda);
-#pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) s[jj] = fmaf(x, __ldg(Bp + p * kNT + jj), s[jj]);
+                    for (int jj = 0; jj < 32; ++jj) redo |= jj < cols && fabsf(v[jj]) < least;
                 }
+                redo = redo && i < a.m;
+                const unsigned rows = __ballot_sync(0xffffffffu, redo);
+                if (rows != 0u) {
+                    float w[32];
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj)
-                    if (redo) v[jj] = s[jj];
+                    for (int jj = 0; jj < 32; ++jj) w[jj] = v[jj];
+                    redo_rows(static_cast<const float *>(a.A) + mt * BM + (warp & 3) * 32, a.lda, a.k,
+                              static_cast<const float *>(a.Bp) + t * a.kp * kNT + half * 32, rows, w);
+#pragma unroll
+                    for (int jj = 0; jj < 32; ++jj) v[jj] = w[jj];
+                }
             }
             const int st = (int)(q % CS);
             const uint32_t par = (uint32_t)((q / CS) & 1);
@@ -458,14 +519,14 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 size_t rank_tc_bytes(int64_t k, int64_t ntiles) {
-    return (size_t)ntiles * (size_t)(k <= kKB ? 1 : 2) * (kBCHUNK + sizeof(uint32_t));
+    return (size_t)ntiles * (size_t)(k <= kKB ? 1 : 2) * (kBCHUNK + sizeof(uint2));
 }
 
 cudaError_t launch_pack_b_rank_tc(int64_t k, int64_t n, const float *B, int64_t ldb, int64_t ntiles, void *dst, cudaStream_t s) {
     const int kc = k <= kKB ? 1 : 2;
     unsigned char *d = static_cast<unsigned char *>(dst);
     pack_b_rank_tc_kernel<<<dim3((unsigned)ntiles, (unsigned)kc), 256, 0, s>>>(
-        B, k, n, ldb, d, reinterpret_cast<uint32_t *>(d + ntiles * kc * kBCHUNK));
+        B, k, n, ldb, d, reinterpret_cast<uint2 *>(d + ntiles * kc * kBCHUNK));
     return cudaGetLastError();
 }
 
@@ -479,7 +540,7 @@ static cudaError_t launch_rank_tc_t(const CUtensorMap *tmA, const CUtensorMap *t
     const int64_t slots = a.num_sms > 0 ? a.num_sms : 1;
     const unsigned grid = (unsigned)(tiles < slots ? tiles : slots);
     if (grid == 0) return cudaSuccess;
-    a.bmin = reinterpret_cast<const uint32_t *>(static_cast<const unsigned char *>(a.Bt) + ntiles * KC * kBCHUNK);
+    a.brange = reinterpret_cast<const uint2 *>(static_cast<const unsigned char *>(a.Bt) + ntiles * KC * kBCHUNK);
     CUtensorMap none;
     std::memset(&none, 0, sizeof(none));
     rankk_tc_kernel<KC><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(*tmA, tmC ? *tmC : none, a, status, tmC ? 1 : 0);

@@ -8,7 +8,7 @@ from gpu_util import assert_parity, run
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(300, 20, 700), (300, 64, 5000), (261, 48, 64)]
+SHAPES = [(300, 20, 700), (300, 64, 5000), (261, 48, 64), (300, 200, 50), (300, 97, 128)]  # regime (i), regime (ii)
 
 
 def draw(m, n, k):
