@@ -18,8 +18,8 @@
 // entry much smaller than its row's or column's largest is thus held with fewer bits than FP64 has: the error is that of
 // the row's and column's scale, not of each product's own, and the guard below bounds what that may cost.
 //
-// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.56 ms (FP64 pipe 98 % busy before; now 39 TFLOP/s FP64,
-// 2.4 TB/s), n = 48: 3.20 ms, n = 32: 55.7 -> 2.48 ms, n = 4: 7.0 -> 1.98 ms (4.3 TB/s); relative error against compensated
+// Measured, m = k = 32768, calls back to back: n = 64: 111.6 -> 3.55 ms (FP64 pipe 98 % busy before; now 40 TFLOP/s FP64,
+// 2.4 TB/s), n = 48: 3.25 ms, n = 32: 55.7 -> 2.48 ms, n = 4: 7.0 -> 2.00 ms (4.3 TB/s); relative error against compensated
 // sums, k = 2048 and 8192: uniform entries 2.8e-16 to 5.5e-16 -> 1.2e-16 to 1.9e-16, rows of B scaled by 10^U[-3,3] 3.0e-16
 // to 5.5e-16 -> 1.3e-16 to 1.8e-16, columns of A scaled by 2^U[-2,2] and rows of B by the inverse 2.8e-16 to 5.5e-16 ->
 // 2.0e-16 to 2.4e-16.
@@ -75,7 +75,8 @@ struct TallTc64Cfg {
     static_assert(F_BYTES >= 2 * kFmaRows * W * 8, "fallback rows");
     static constexpr int OFF_BAR = OFF_F + F_BYTES;
     static constexpr int NBAR = 2 * SA + 2 * SB + 18;
-    static constexpr int SMEM = OFF_BAR + NBAR * 8 + 96;
+    static constexpr int OFF_Z = OFF_BAR + NBAR * 8 + 96;     // rows taken as zero
+    static constexpr int SMEM = OFF_Z + BM;
     static constexpr int THREADS = 640;                       // 96 registers each at launch, dealt out again by role:
     static constexpr int CREG = W == 64 ? 72 : 80, PREG = W == 64 ? 144 : W == 48 ? 128 : 112;
     static constexpr int MREG = W == 64 ? 48 : W == 48 ? 64 : 96;
@@ -120,6 +121,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
     unsigned *abort_flag = tslot + 2;
     unsigned *unsafe = tslot + 3;
     unsigned *gslot = tslot + 4;       // [2] step of rowE that holds a group's scales
+    unsigned char *zrow = smem + Cfg::OFF_Z;  // [BM] no nonzero entry in the guard's columns: zero unless the converters see one
     volatile unsigned *gnew = tslot + 8;  // [4] steps: a byte per quarter of the rows, set where scales grew: a new group
 
     const int warp = threadIdx.x / 32;
@@ -159,6 +161,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         *unsafe = 0u;
         fence_mbar_init();
     }
+    if (threadIdx.x < BM / 4) reinterpret_cast<unsigned *>(zrow)[threadIdx.x] = 0u;
     if (warp == 17) tc_alloc(tslot, Cfg::TMEM_COLS);
     tcf_before();
     __syncthreads();
@@ -387,6 +390,9 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         const int ldv = (int)((uint64_t)a.lda & 1);
         const uint32_t vmask = row < a.m ? 0xffffffffu : 0u;  // rows beyond m count as zeros
         uint64_t *sbar = &scale[warp & 3];
+        // for rows taken as zero: the bits of their entries (W = 16: while no scale has counted any, which costs n = 4 1 %;
+        // without that branch 1.4 %, above W = 16 the branch costs more)
+        uint32_t seen_lo = 0u, seen_hi = 0u;
         bool ok = true;
         const int steps = __all_sync(0xffffffffu, go()) ? iters : 0;
         for (int it = warp / 4; it < steps; it += 2) {
@@ -410,7 +416,13 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             __syncwarp();
             if (lane == 0) mbar_arrive(&aempty[s]);
 #pragma unroll
-            for (int q = 0; q < KB; q += 2) mx = __vimax3_s32(mx, (int)tc64_abs(hi[q]), (int)tc64_abs(hi[q + 1]));
+            for (int q = 0; q < KB; q += 2) {
+                mx = __vimax3_s32(mx, (int)tc64_abs(hi[q]), (int)tc64_abs(hi[q + 1]));
+                if constexpr (W > 16) {
+                    seen_lo |= lo[q] | lo[q + 1];
+                    seen_hi |= hi[q] | hi[q + 1];
+                }
+            }
             mx >>= 20;
             // the row's scale after the step before, and after this one
             int E = kTc64Emin;
@@ -428,6 +440,12 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
                 reinterpret_cast<volatile unsigned char *>(gnew)[(it & 3) * 4 + (warp & 3)] = grown ? 1 : 0;
             __syncwarp();
             if (lane == 0) mbar_arrive(sbar);
+            if constexpr (W == 16) {
+                if (E == kTc64Emin) {
+#pragma unroll
+                    for (int q = 0; q < KB; ++q) seen_lo |= hi[q] << 1 | lo[q];
+                }
+            }
             uint32_t sgn[KB / 2];
 #pragma unroll
             for (int q = 0; q < KB; q += 2) sgn[q / 2] = tc64_sign2(hi[q], hi[q + 1]);
@@ -493,6 +511,7 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
             atomicOr(a.status, kDevErrTimeout);
             atomicOr(abort_flag, 1u);
         }
+        if (zrow[r] != 0 && (seen_hi << 1 | seen_lo) != 0u) *unsafe = 1u;
         named_barrier(1, 512);  // the promoters read the last scales after it
         if (*abort_flag != 0u || a.splits == 1) return;
         finish();
@@ -563,11 +582,11 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         }
         release_reads_to_async_copy();  // the fallback's copies may follow
         if (bound < need) {
-            // too small: fmas, unless the row is zero throughout
-            const uint64_t *rp = static_cast<const uint64_t *>(a.A) + row;
-            uint64_t any = 0;
-            for (int64_t p = k0; p < k1 && p < a.k && any == 0; ++p) any = __ldg(rp + p * a.lda) << 1;
-            if (any != 0) *unsafe = 1u;
+            // Too small: fmas, unless the row is zero throughout, which the converters know at the end (a scan of the row
+            // here held the block up for 0.4 us a column: m = k = 16384, n = 4 with one zero row in every slab 6.58 ms, 0.55
+            // so, 0.53 without; every other row zero 0.58).
+            if (E0 == 0) zrow[r] = 1;
+            else *unsafe = 1u;
             bound = 0x7fffffff, E0 = kTc64Emax;
         }
         if ((E0 < kTc64Emin && row < a.m && bound != 0x7fffffff) || bad_b != 0u) *unsafe = 1u;
@@ -657,9 +676,10 @@ __device__ __forceinline__ void tall_tc64_block(const CUtensorMap *tmA, const Ta
         atomicOr(abort_flag, 1u);
     }
     if (started && row < a.m) {
-        // infinities and NaNs, rows wholly below the scales, and a row that grew after its guard columns
+        // infinities and NaNs, rows wholly below the scales, rows taken as zero that are not, and a row that grew after its
+        // guard columns
         const int sft = E - E0;
-        if (E > kTc64Emax || (E == kTc64Emin && bound != 0x7fffffff) ||
+        if (E > kTc64Emax || (E == kTc64Emin && bound != 0x7fffffff) || (E != kTc64Emin && zrow[r] != 0) ||
             (bound != 0x7fffffff && (sft > 30 || (bound >> max(sft, 0)) < need)))
             *unsafe = 1u;
     }
