@@ -236,19 +236,20 @@ tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k
     pb->tc_data = nullptr;
     pb->tc_min = nullptr;
     if (pb->bytes > 0) {
-        const bool tc = tc_pack(dtype, regime, precision, n, k);
+        bool tc = tc_pack(dtype, regime, precision, n, k);
         const size_t off = (size_t)round_up((int64_t)pb->bytes, 256);
         const size_t pieces = (size_t)pb->kp * (size_t)tc_width(n) * 6;
-        const bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
+        bool tc64 = precision == TSMM_PREC_NATIVE && tc64_pack(dtype, regime, n, k);
         bool rtc = rank_tc(dtype, regime, precision, k), rtc64 = rank_tc64(dtype, regime, precision, k);
-        cudaError_t e = cudaMalloc(&pb->data, tc      ? off + pieces + (size_t)(pb->kp / kTcKB) * 2 * sizeof(float)
-                                              : tc64  ? off + tc64_bytes(k, n)
-                                              : rtc   ? off + rank_tc_bytes(k, pb->ntiles)
-                                              : rtc64 ? off + rank_tc64_bytes(k, pb->ntiles)
-                                                      : pb->bytes);
-        if (e != cudaSuccess && (rtc || rtc64)) {  // the panel alone serves the fma kernels
+        const size_t more = tc      ? pieces + (size_t)(pb->kp / kTcKB) * 2 * sizeof(float)
+                            : tc64  ? tc64_bytes(k, n)
+                            : rtc   ? rank_tc_bytes(k, pb->ntiles)
+                            : rtc64 ? rank_tc64_bytes(k, pb->ntiles)
+                                    : 0;
+        cudaError_t e = cudaMalloc(&pb->data, more ? off + more : pb->bytes);
+        if (e != cudaSuccess && more) {  // the panel alone serves the fma kernels
             cudaGetLastError();
-            rtc = rtc64 = false;
+            tc = tc64 = rtc = rtc64 = false;
             e = cudaMalloc(&pb->data, pb->bytes);
         }
         if (e != cudaSuccess) {
@@ -547,20 +548,26 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
     a.bmin = pb->tc_min;
     a.arows = 0;
 
-    // A tensor-core plan too short in k for it: the fma kernel on its own slabs (one split: no workspace); the blocks' own
-    // fma path, which grouped launches take, gives the same bits (m = 100000, n = 64, k = 8: 12 us, 50 on the blocks' own)
-    const bool short_k = p->tc && p->dtype == TSMM_F32 && k < kTcMinK;
-    const int bm = short_k ? tall_bm(p->dtype, p->np) : p->bm;
-    if (short_k) a.slabs = (m + bm - 1) / bm;
+    // A tensor-core plan whose B was packed without its tensor-core form (for lack of memory), or too short in k for it: the
+    // fma kernel on its own slabs, in one split, which needs no workspace.  (The blocks' own fma path, which grouped launches
+    // with few columns take, gives the same bits there; m = 100000, n = 64, k = 8: 12 us, 50 on that path.)
+    const bool tc = p->tc && pb->tc_data && !(p->dtype == TSMM_F32 && k < kTcMinK);
+    const bool fma = p->tc && !tc;
+    const int bm = fma ? tall_bm(p->dtype, p->np) : p->bm;
+    if (fma) {
+        a.slabs = (m + bm - 1) / bm;
+        a.splits = 1;
+        a.kchunk = a.kp;
+    }
 
     const bool tma = aligned(A_dev, 16) && ((lda * (int64_t)es) % 16 == 0) && m < INT_MAX &&
                      k < INT_MAX && (lda * (int64_t)es) < (1LL << 40) && encoder() != nullptr;
-    if (tma && (p->tmap_ptr != A_dev || p->tmap_lda != lda)) {
+    if (tma && (p->tmap_ptr != A_dev || p->tmap_lda != lda || p->tmap_tc != tc)) {
         // box: bm rows x 32 columns (the regime (i) stage and the regime (ii) k chunk)
         const cuuint64_t gdim[2] = {(cuuint64_t)m, (cuuint64_t)k};
         const cuuint64_t gstride[1] = {(cuuint64_t)(lda * (int64_t)es)};
         const cuuint32_t box[2] = {(cuuint32_t)bm,
-                                   (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k, p->tc)};
+                                   (cuuint32_t)a_box_k(p->dtype, p->regime, p->precision, p->k, tc)};
         const cuuint32_t estr[2] = {1, 1};
         CUresult r = encoder()(&p->tmap,
                                p->dtype == TSMM_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -575,6 +582,7 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         }
         p->tmap_ptr = A_dev;
         p->tmap_lda = lda;
+        p->tmap_tc = tc;
     }
     if (p->precision == TSMM_PREC_BF16X3) {
         if (p->regime == 2) {
@@ -689,12 +697,12 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
         if (scratch) cudaFreeAsync(scratch, s);  // after the kernel, in stream order
         return cuda_status(e);
     }
-    const bool tc = p->tc && !short_k;
     if (tc && !tma) {
-        if (p->tmap_ptr != A_dev || p->tmap_lda != lda) {
+        if (p->tmap_ptr != A_dev || p->tmap_lda != lda || p->tmap_tc != tc) {
             p->arows = encode_a_rows(&p->tmap, p->dtype, A_dev, m, k, lda);
             p->tmap_ptr = A_dev;
             p->tmap_lda = lda;
+            p->tmap_tc = tc;
         }
         a.arows = p->arows;
     }

@@ -77,6 +77,7 @@ int group_kind(const tsmm_group_item &it) {
     if (!(p->regime == 1 && p->precision == TSMM_PREC_NATIVE && p->m > 0 && p->n > 0 && p->k > 0 && !alpha_zero &&
           p->m < INT_MAX && p->k < INT_MAX && p->slabs * (int64_t)p->splits < INT_MAX))
         return 0;
+    if (p->tc && !it.pb->tc_data) return 0;  // packed without its tensor-core form, for lack of memory
     const bool tma = is_aligned(it.A_dev, 16) && (it.lda * (int64_t)es) % 16 == 0 &&
                      (it.lda * (int64_t)es) < (1LL << 40) && encoder_grouped() != nullptr;
     return tma ? 1 : 2;

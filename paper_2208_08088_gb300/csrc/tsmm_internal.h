@@ -183,6 +183,7 @@ struct tsmm_plan_s {
     // one-entry caches of the TMA descriptors for A and (regime (ii)) C
     const void *tmap_ptr;
     int64_t tmap_lda;
+    bool tmap_tc;              // the tensor-core kernel's map (the fma kernel's has other boxes)
     CUtensorMap tmap;
     int64_t arows;             // tmap is encode_a_rows' with so many rows (tensor-core kernels, unaligned A)
     const void *tmapc_ptr;
