@@ -296,7 +296,11 @@ TSMM_API tsmm_status tsmm_autotune(int64_t m, int64_t n, int64_t k, tsmm_dtype d
  * The plan cache (the install-time record of tuned choices).  Text format, one
  * entry per line: `f32|f64 m n k sm_count splits` for an exact m, or
  * `f32q|f64q b n k sm_count splits` for every m of quarter-octave bucket b
- * (b = floor(4 log2 m)); lines starting with '#' are comments.  If the environment variable TSMM_PLAN_CACHE names a file, it is
+ * (b = floor(4 log2 m)); lines starting with '#' are comments.  Entries after a
+ * line that starts with `# tsmm plan cache v3` (save writes it) were tuned with
+ * the tensor-core kernels; others are kept, but not used for shapes that run on
+ * those, whose stages and slabs differ from the kernels they were tuned for.
+ * If the environment variable TSMM_PLAN_CACHE names a file, it is
  * loaded on first use.  load merges a file into the cache (INVALID_ARG if the
  * file is missing or malformed, leaving the cache unchanged); save writes the
  * whole cache; clear empties it; size returns the number of entries (exact

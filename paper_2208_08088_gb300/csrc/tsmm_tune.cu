@@ -7,11 +7,14 @@
 // SM count) -- and by (dtype, quarter-octave bucket of m, n, k, SM count), so a
 // tuned choice also serves the other m of its bucket -- that tsmm_plan
 // consults, and that can be saved to and loaded from a text file
-// (TSMM_PLAN_CACHE names one to load on first use).
+// (TSMM_PLAN_CACHE names one to load on first use).  A file says which kernels its
+// counts were tuned for: those from before the tensor-core kernels are kept, but
+// not used for shapes that now run there, whose stages and slabs differ.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <new>
@@ -30,8 +33,14 @@ namespace {
 using Key = std::tuple<int, int64_t, int64_t, int64_t, int>;
 
 std::mutex g_cache_mu;
-std::map<Key, int> g_cache;   // exact m
-std::map<Key, int> g_bucket;  // m replaced by its bucket
+struct Entry {
+    int splits;
+    bool fma_only;  // tuned before the tensor-core kernels: from a file without kFileMark
+};
+std::map<Key, Entry> g_cache;   // exact m
+std::map<Key, Entry> g_bucket;  // m replaced by its bucket
+constexpr char kFileMark[] = "# tsmm plan cache v3";     // heads the entries tuned with the tensor-core kernels
+constexpr char kOldFileMark[] = "# tsmm plan cache v2";  // ... and without
 bool g_env_loaded = false;
 
 // quarter-octave bucket of m >= 1: floor(4 log2 m); 2^(b/4) <= m < 2^((b+1)/4)
@@ -43,9 +52,11 @@ tsmm_status load_file_locked(const char *path) {
     FILE *f = std::fopen(path, "r");
     if (!f) return TSMM_ERR_INVALID_ARG;
     char line[512];
-    std::map<Key, int> parsed, parsed_b;
-    bool bad = false;
+    std::map<Key, Entry> parsed, parsed_b;
+    bool bad = false, fma_only = true;
     while (std::fgets(line, sizeof line, f)) {
+        if (std::strncmp(line, kFileMark, sizeof kFileMark - 1) == 0) fma_only = false;
+        if (std::strncmp(line, kOldFileMark, sizeof kOldFileMark - 1) == 0) fma_only = true;
         if (line[0] == '#' || line[0] == '\n' || line[0] == '\0') continue;
         char dt[8] = {0};
         long long m, n, k;
@@ -66,12 +77,24 @@ tsmm_status load_file_locked(const char *path) {
             bad = true;
             break;
         }
-        (bucket ? parsed_b : parsed)[Key(d, m, n, k, sms)] = splits;
+        (bucket ? parsed_b : parsed)[Key(d, m, n, k, sms)] = Entry{splits, fma_only};
     }
     std::fclose(f);
     if (bad) return TSMM_ERR_INVALID_ARG;
-    for (auto &kv : parsed) g_cache[kv.first] = kv.second;
-    for (auto &kv : parsed_b) g_bucket[kv.first] = kv.second;
+    auto merge = [](std::map<Key, Entry> &to, const std::map<Key, Entry> &from) {
+        for (auto &kv : from) {
+            auto it = to.find(kv.first);
+            const tsmm_dtype d = static_cast<tsmm_dtype>(std::get<0>(kv.first));
+            const int64_t n = std::get<2>(kv.first), k = std::get<3>(kv.first);
+            // an entry that a tensor-core shape cannot use does not replace one that it can
+            if (it != to.end() && kv.second.fma_only && !it->second.fma_only &&
+                (tc_pack(d, regime_of(k, n), TSMM_PREC_NATIVE, n, k) || tc64_pack(d, regime_of(k, n), n, k)))
+                continue;
+            to[kv.first] = kv.second;
+        }
+    };
+    merge(g_cache, parsed);
+    merge(g_bucket, parsed_b);
     return TSMM_OK;
 }
 
@@ -89,17 +112,20 @@ namespace tsmm {
 int plan_cache_lookup(tsmm_dtype dtype, int64_t m, int64_t n, int64_t k, int sms) {
     std::lock_guard<std::mutex> lock(g_cache_mu);
     load_env_once_locked();
+    const int regime = regime_of(k, n);
+    const bool tc = tc_pack(dtype, regime, TSMM_PREC_NATIVE, n, k) || tc64_plan(dtype, regime, m, n, k);
+    auto usable = [&](const Entry &e) { return !(tc && e.fma_only); };
     auto it = g_cache.find(Key(dtype, m, n, k, sms));
-    if (it != g_cache.end()) return it->second;
+    if (it != g_cache.end() && usable(it->second)) return it->second.splits;
     auto ib = g_bucket.find(Key(dtype, m_bucket(m), n, k, sms));
-    return ib == g_bucket.end() ? 0 : ib->second;
+    return ib == g_bucket.end() || !usable(ib->second) ? 0 : ib->second.splits;
 }
 
 void plan_cache_store(tsmm_dtype dtype, int64_t m, int64_t n, int64_t k, int sms, int splits) {
     std::lock_guard<std::mutex> lock(g_cache_mu);
     load_env_once_locked();
-    g_cache[Key(dtype, m, n, k, sms)] = splits;
-    g_bucket[Key(dtype, m_bucket(m), n, k, sms)] = splits;
+    g_cache[Key(dtype, m, n, k, sms)] = Entry{splits, false};
+    g_bucket[Key(dtype, m_bucket(m), n, k, sms)] = Entry{splits, false};
 }
 
 }  // namespace tsmm
@@ -118,17 +144,18 @@ tsmm_status tsmm_plan_cache_save(const char *path) {
     std::lock_guard<std::mutex> lock(g_cache_mu);
     FILE *f = std::fopen(path, "w");
     if (!f) return TSMM_ERR_INVALID_ARG;
-    std::fprintf(f, "# tsmm plan cache v2: dtype m n k sm_count splits (dtype f32q/f64q: m is a "
-                    "quarter-octave bucket)\n");
-    for (auto &kv : g_cache) {
-        std::fprintf(f, "%s %lld %lld %lld %d %d\n", std::get<0>(kv.first) == TSMM_F64 ? "f64" : "f32",
-                     (long long)std::get<1>(kv.first), (long long)std::get<2>(kv.first),
-                     (long long)std::get<3>(kv.first), std::get<4>(kv.first), kv.second);
-    }
-    for (auto &kv : g_bucket) {
-        std::fprintf(f, "%s %lld %lld %lld %d %d\n", std::get<0>(kv.first) == TSMM_F64 ? "f64q" : "f32q",
-                     (long long)std::get<1>(kv.first), (long long)std::get<2>(kv.first),
-                     (long long)std::get<3>(kv.first), std::get<4>(kv.first), kv.second);
+    auto write = [&](const std::map<Key, Entry> &entries, const char *f32, const char *f64, bool fma_only) {
+        for (auto &kv : entries)
+            if (kv.second.fma_only == fma_only)
+                std::fprintf(f, "%s %lld %lld %lld %d %d\n", std::get<0>(kv.first) == TSMM_F64 ? f64 : f32,
+                             (long long)std::get<1>(kv.first), (long long)std::get<2>(kv.first),
+                             (long long)std::get<3>(kv.first), std::get<4>(kv.first), kv.second.splits);
+    };
+    for (const bool fma_only : {true, false}) {
+        std::fprintf(f, "%s: dtype m n k sm_count splits (dtype f32q/f64q: m is a quarter-octave bucket)%s\n",
+                     fma_only ? kOldFileMark : kFileMark, fma_only ? "; tuned before the tensor-core kernels" : "");
+        write(g_cache, "f32", "f64", fma_only);
+        write(g_bucket, "f32q", "f64q", fma_only);
     }
     const bool ok = std::fclose(f) == 0;
     return ok ? TSMM_OK : TSMM_ERR_INVALID_ARG;
