@@ -182,12 +182,14 @@ tsmm_status tsmm_autotune(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, con
     tsmm_plan_t base = nullptr;
     tsmm_status st = create_plan(m, n, k, dtype, 0, &base);
     if (st != TSMM_OK) return st;
-    if (base->regime != 1 || m == 0 || n == 0 || k == 0 || base->kp / kTallBKS <= 1) {
+    // stages of k that a split is cut into (plan_layout): 64 columns for the FP64 tensor-core kernel
+    const int64_t stage = base->tc && dtype == TSMM_F64 ? 64 : kTallBKS;
+    const int64_t kstages = (base->kp + stage - 1) / stage;
+    if (base->regime != 1 || m == 0 || n == 0 || k == 0 || kstages <= 1) {
         *out = base;  // nothing to tune: one split is the only choice
         return TSMM_OK;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int64_t kstages = base->kp / kTallBKS;
     const int sms = base->num_sms;
     // candidate split counts: the model's choice for 1..4 resident blocks per
     // SM, its halves and doubles, no split, and counts that fill whole waves
@@ -204,9 +206,12 @@ tsmm_status tsmm_autotune(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, con
         const int64_t want = (int64_t)waves * resident * sms;
         cand.insert(std::max<int64_t>(1, want / std::max<int64_t>(1, base->slabs)));
     }
+    // counts that cut k alike are one plan
     std::vector<int64_t> cands;
+    std::set<int64_t> chunks;
+    if (base->splits > 0) chunks.insert((kstages + base->splits - 1) / base->splits), cands.push_back(base->splits);
     for (int64_t c : cand)
-        if (c >= 1 && c <= kstages && c <= 65535) cands.push_back(c);
+        if (c >= 1 && c <= kstages && c <= 65535 && chunks.insert((kstages + c - 1) / c).second) cands.push_back(c);
 
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
