@@ -40,14 +40,18 @@
  *     aborts or throws; every failure is a status code.
  *   - Accuracy: every entry satisfies |C - C_exact| <= 4*k*u*(|alpha| sum_p
  *     |A[i,p]||B[p,j]| + |beta||C0[i,j]|) with u = 2^-24 (F32) / 2^-53 (F64).
- *     Products are accumulated with IEEE fma in the working precision, or on the
- *     tensor cores from splits of every entry (errors measured smaller than the
- *     fma chain's): F32 with 16 < n <= 64, or with n > 64 and k > 32, from exact
- *     splits into three BF16 values with all products down to 2^-25 of |a||b|;
- *     F64 with 1 < n <= 64 and 256 <= k <= 2^20, or with n > 64 and k >= 4, from
- *     55- to 63-bit fixed point cut into 8-bit digits whose products are summed
- *     exactly.  Inputs such a split cannot carry within the
- *     bound (infinities, NaNs, overflow, extreme or very unevenly scaled
+ *     Products are accumulated with IEEE fma in the working precision, or, unless
+ *     the plan's arithmetic is TSMM_PREC_FMA, on the tensor cores from splits of
+ *     every entry: F32 with 16 < n <= 64 and k >= 16, or with n > 64 and k > 32,
+ *     from exact splits into three BF16 values with all products down to 2^-25 of
+ *     |a||b|; F64 with 1 < n <= 64 and 256 <= k <= 2^20, or with n > 64 and
+ *     k >= 4, from 55- to 63-bit fixed point below the largest entry of each row
+ *     of A and column of B, cut into 8-bit digits whose products are summed
+ *     exactly.  Errors are measured smaller than the fma chain's on entries of one
+ *     size and on rows of A and B scaled by up to 10^+-3; F64 entries far below
+ *     their row's or column's largest are held with fewer bits than the fma chain
+ *     has for them.  Inputs that cannot be carried within the bound (infinities,
+ *     NaNs, overflow, sums too small for their terms, very unevenly scaled
  *     entries) are found by the kernel and computed with fma.
  */
 #ifndef TSMM_H
@@ -80,8 +84,10 @@ typedef enum {
 } tsmm_status;
 
 /*
- * Arithmetic of a plan / packed B.  NATIVE: IEEE fma in the working precision
- * (the contract stated above).  BF16X3 (TSMM_F32, both regimes): the
+ * Arithmetic of a plan / packed B.  NATIVE: the contract stated above.  FMA: the
+ * same with IEEE fma in the working precision throughout (the FMA pipes; no
+ * tensor core, at their speed; grouped launches run such problems one by one).
+ * BF16X3 (TSMM_F32, both regimes): the
  * tensor-core mode C = alpha*(A_hi*B_hi + A_hi*B_lo + A_lo*B_hi) + beta*C0
  * with x_hi = bf16(x), x_lo = bf16(x - x_hi) and FP32 accumulation in tensor
  * memory (tcgen05.mma).  It drops A_lo*B_lo and the split residues, about
@@ -92,7 +98,7 @@ typedef enum {
  * aligned to 4 bytes: an A that a tensor map cannot describe (base or lda*4
  * not a multiple of 16) is moved column by column, with the same result.
  */
-typedef enum { TSMM_PREC_NATIVE = 0, TSMM_PREC_BF16X3 = 1 } tsmm_precision;
+typedef enum { TSMM_PREC_NATIVE = 0, TSMM_PREC_BF16X3 = 1, TSMM_PREC_FMA = 2 } tsmm_precision;
 
 typedef void *tsmm_stream_t; /* a cudaStream_t */
 typedef struct tsmm_packed_b_s *tsmm_packed_b;

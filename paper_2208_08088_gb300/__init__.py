@@ -25,7 +25,7 @@ import os
 from . import build as _build
 
 __all__ = [
-    "TsmmError", "F32", "F64", "PREC_NATIVE", "PREC_BF16X3", "lib", "library_path",
+    "TsmmError", "F32", "F64", "PREC_NATIVE", "PREC_BF16X3", "PREC_FMA", "lib", "library_path",
     "tsmm_pack_b_ex", "tsmm_plan_ex",
     "tsmm_status_string", "tsmm_version", "tsmm_pack_b", "tsmm_packed_b_destroy",
     "tsmm_packed_b_info", "tsmm_packed_b_read", "tsmm_plan", "tsmm_plan_destroy", "tsmm_plan_info", "tsmm_execute",
@@ -41,7 +41,7 @@ __all__ = [
 ]
 
 F32, F64 = 0, 1
-PREC_NATIVE, PREC_BF16X3 = 0, 1
+PREC_NATIVE, PREC_BF16X3, PREC_FMA = 0, 1, 2
 DIAG_FFMA, DIAG_FFMA2, DIAG_DFMA, DIAG_DMMA = 0, 1, 2, 3
 STATUS = {
     0: "TSMM_OK", 1: "TSMM_ERR_INVALID_ARG", 2: "TSMM_ERR_UNSUPPORTED_SHAPE",

@@ -35,6 +35,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
 
 bool valid_dtype(tsmm_dtype d) { return d == TSMM_F32 || d == TSMM_F64; }
 
+bool valid_precision(tsmm_precision p, tsmm_dtype d) {
+    return p == TSMM_PREC_NATIVE || p == TSMM_PREC_FMA || (p == TSMM_PREC_BF16X3 && d == TSMM_F32);
+}
+
 bool aligned(const void *p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
 thread_local const char *g_last_cuda_error = "no error";
@@ -197,8 +201,7 @@ tsmm_status tsmm_pack_b(tsmm_dtype dtype, int64_t k, int64_t n, const void *B_de
 tsmm_status tsmm_pack_b_ex(tsmm_dtype dtype, tsmm_precision precision, int64_t k, int64_t n,
                            const void *B_dev, int64_t ldb, tsmm_stream_t stream, tsmm_packed_b *out) {
     if (!out || !valid_dtype(dtype) || k < 0 || n < 0) return TSMM_ERR_INVALID_ARG;
-    if (precision != TSMM_PREC_NATIVE && precision != TSMM_PREC_BF16X3) return TSMM_ERR_INVALID_ARG;
-    if (precision == TSMM_PREC_BF16X3 && dtype != TSMM_F32) return TSMM_ERR_INVALID_ARG;
+    if (!valid_precision(precision, dtype)) return TSMM_ERR_INVALID_ARG;
     if (ldb < std::max<int64_t>(1, k)) return TSMM_ERR_INVALID_ARG;
     if (k > 0 && n > 0 && !B_dev) return TSMM_ERR_INVALID_ARG;
     const size_t es = dtype_size(dtype);
@@ -330,8 +333,7 @@ tsmm_status tsmm_plan(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, tsmm_pl
 tsmm_status tsmm_plan_ex(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, tsmm_precision precision,
                          tsmm_plan_t *out) {
     if (!out || !valid_dtype(dtype) || m < 0 || n < 0 || k < 0) return TSMM_ERR_INVALID_ARG;
-    if (precision != TSMM_PREC_NATIVE && precision != TSMM_PREC_BF16X3) return TSMM_ERR_INVALID_ARG;
-    if (precision == TSMM_PREC_BF16X3 && dtype != TSMM_F32) return TSMM_ERR_INVALID_ARG;
+    if (!valid_precision(precision, dtype)) return TSMM_ERR_INVALID_ARG;
     int dev = current_device();
     int sms = 0;
     if (dev >= 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -438,7 +440,8 @@ tsmm_status plan_layout(int64_t m, int64_t n, int64_t k, tsmm_dtype dtype, int f
         }
     } else if (regime == 1) {
         p->np = tall_np(n);
-        p->tc = tc_pack(dtype, regime, precision, n, k) || tc64_plan(dtype, regime, m, n, k);
+        p->tc = tc_pack(dtype, regime, precision, n, k) ||
+                (precision == TSMM_PREC_NATIVE && tc64_plan(dtype, regime, m, n, k));
         // k split in stages of kTallBKS columns; the FP64 guard looks at aligned windows of 64
         const int64_t stage = p->tc && dtype == TSMM_F64 ? 64 : kTallBKS;
         p->bm = p->tc ? kTcRows : tall_bm(dtype, p->np);
@@ -687,9 +690,9 @@ tsmm_status tsmm_execute(tsmm_plan_t p, double alpha, const void *A_dev, int64_t
                 return st;
             }
         }
-        // (a B packed without its tensor-core form, for lack of memory, is left to the plain-load kernel: the fma
-        // kernels' tensor copies serve k < kRankTcMinK)
-        const bool plain = !rtc && rank_tc(p->dtype, p->regime, p->precision, k);
+        // (without the tensor cores, by choice or a B packed without its form for lack of memory, FP32 is left to the
+        // plain-load kernel here: the fma kernels' tensor copies serve k < kRankTcMinK)
+        const bool plain = !rtc && p->dtype == TSMM_F32 && k >= kRankTcMinK;
         const CUtensorMap *ta = tma_a && !plain ? (scratch ? &tm_scratch : &p->tmap) : nullptr;
         const CUtensorMap *tc = tmc && !plain ? &p->tmapc : nullptr;
         const cudaError_t e = rtc ? launch_rankk_tc(ta, tc, ra, p->status, s)

@@ -254,7 +254,7 @@ inline bool rank_tc(tsmm_dtype d, int regime, int precision, int64_t k) {
     return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankTcMinK;
 }
 inline bool rank_wide(tsmm_dtype d, int regime, int precision, int64_t k) {
-    return d == TSMM_F32 && regime == 2 && precision == 0 && k >= kRankWideMinK && k < kRankTcMinK;
+    return d == TSMM_F32 && regime == 2 && precision != TSMM_PREC_BF16X3 && k >= kRankWideMinK && k < kRankTcMinK;
 }
 inline int a_box_k(tsmm_dtype d, int regime, int precision, int64_t k, bool tc) {
     if (tc && d == TSMM_F64) return kTc64KB;
