@@ -200,7 +200,7 @@ __device__ __forceinline__ void tall_finish(T *red, const TallArgs &a, int64_t s
         Vec<T, R> s;
 #pragma unroll
         for (int r = 0; r < R; ++r) s.v[r] = T(0);
-        // the loads of kAhead splits are in flight together (this block's own partial among them: it was published
+        // the loads of up to 8 splits are in flight together (this block's own partial among them: it was published
         // above), the sums taken in order: one load ahead had made this a chain of L2 latencies, half of a small
         // problem's time (m = k = 2048, n = 16, 38 splits: 40 us a call)
         // (groups of 8, then the remainder's 4, 2 and 1, under uniform branches: adds of absent splits, though predicated
@@ -237,6 +237,12 @@ struct AccTile {
         }
     }
     __device__ __forceinline__ T get(int r, int c) const { return v[r][c]; }
+    __device__ __forceinline__ void add(const AccTile &o) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < CN; ++c) v[r][c] += o.v[r][c];
+    }
 };
 
 template <int R, int CN>
@@ -268,6 +274,12 @@ struct AccTilePairs {
     __device__ __forceinline__ float get(int r, int c) const {
         return (c & 1) ? v[r][c / 2].y : v[r][c / 2].x;
     }
+    __device__ __forceinline__ void add(const AccTilePairs &o) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < CN / 2; ++c) v[r][c] = __fadd2_rn(v[r][c], o.v[r][c]);
+    }
 };
 
 template <typename T, int NP>
@@ -280,6 +292,33 @@ struct TallAcc<float, NP> {
     using Cfg = TallCfg<float, NP>;
     using type = typename std::conditional<(Cfg::CN >= 2), AccTilePairs<Cfg::R, Cfg::CN>,
                                            AccTile<float, Cfg::R, Cfg::CN, Cfg::BV>>::type;
+};
+
+// The tile's chains of fmas cut in eight (at least two stages long each), their sums totalled apart, for the FP32 widths up
+// to 16: with few splits their chains are long for their k (m = k = 2048, n = 16 on 8 splits: relative error 2.2e-7 ->
+// 1.3e-7, 18.1 -> 18.4 us; m = k = 32768, n = 16: 8.7e-7 -> 3.1e-7, 633 -> 626 us).
+template <typename T, int NP>
+struct TallTotal {
+    static constexpr bool ON = sizeof(T) == 4 && NP <= 16;
+    typename TallAcc<T, NP>::type tot;
+    int seg, left;
+    __device__ __forceinline__ explicit TallTotal(int iters) {
+        if constexpr (ON) {
+            tot.zero();
+            left = seg = iters > 16 ? iters / 8 : 2;
+        }
+    }
+    __device__ __forceinline__ void stage(typename TallAcc<T, NP>::type &acc) {
+        if constexpr (ON)
+            if (--left == 0) {
+                tot.add(acc);
+                acc.zero();
+                left = seg;
+            }
+    }
+    __device__ __forceinline__ void finish(typename TallAcc<T, NP>::type &acc) {
+        if constexpr (ON) acc.add(tot);
+    }
 };
 
 // One block's work item (m-slab `slab`, k range `split`) with A described by
@@ -349,6 +388,7 @@ __device__ __forceinline__ void tall_tma_block(const CUtensorMap *tmA, const Tal
 
     typename TallAcc<T, NP>::type acc;
     acc.zero();
+    TallTotal<T, NP> total(iters);
 
     bool ok = true;
     for (int it = 0; it < iters; ++it) {
@@ -368,7 +408,9 @@ __device__ __forceinline__ void tall_tma_block(const CUtensorMap *tmA, const Tal
         release_reads_to_async_copy();
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);
+        total.stage(acc);
     }
+    total.finish(acc);
     if (!ok && lane == 0) {
         atomicOr(a.status, kDevErrTimeout);
         atomicOr(abort_flag, 1u);
@@ -551,6 +593,7 @@ __device__ __forceinline__ void tall_async_block(const TallArgs &a, int64_t slab
     const int cloc = g * Cfg::CN;
     typename TallAcc<T, NP>::type acc;
     acc.zero();
+    TallTotal<T, NP> total(iters);
     // every stage starts at a multiple of BKS (k splits are whole stages), so a
     // column's offset within 16 bytes depends only on its index mod V
     int doff[V];
@@ -583,7 +626,9 @@ __device__ __forceinline__ void tall_async_block(const TallArgs &a, int64_t slab
         release_reads_to_async_copy();
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);
+        total.stage(acc);
     }
+    total.finish(acc);
     if (!ok && lane == 0) {
         atomicOr(a.status, kDevErrTimeout);
         atomicOr(abort_flag, 1u);
