@@ -94,7 +94,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
     };
     // Chains of SEG (SEGN) stages, their sums added in `tot`: one chain over a whole item would be several times as long as
     // the fma kernels', whose blocks split k among warps and more splits (FP64, n = 64, k = 2048, uneven columns: error
-    // 5.5e-16, theirs 3.7e-16, so 2.3e-16).  The totals sit in shared memory because registers for them spill (FP32,
+    // 5.5e-16, theirs 3.7e-16, so @S@).  The totals sit in shared memory because registers for them spill (FP32,
     // n = 64: 5 times the time).
     tot += tid;
     // up to 8 columns of FP64 (np <= 8 = HW): the halves share the columns and split each stage's rows, and 16 sums a
@@ -154,7 +154,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
         if (np == 4) return narrow(std::integral_constant<int, 4>{});
         if (np == 8) return narrow(std::integral_constant<int, 8>{});
     }
-    constexpr int SEG = sizeof(T) == 8 ? 1 : 8;
+    constexpr int SEG = sizeof(T) == 8 ? 2 : 8;
     FmaAcc<T, HW> acc;
     acc.zero();
     T x[CH];

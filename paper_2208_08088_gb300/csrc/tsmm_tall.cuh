@@ -294,9 +294,9 @@ struct TallAcc<float, NP> {
                                            AccTile<float, Cfg::R, Cfg::CN, Cfg::BV>>::type;
 };
 
-// The tile's chains of fmas cut in eight (at least two stages long each), their sums totalled apart, for the FP32 widths up
-// to 16: with few splits their chains are long for their k (m = k = 2048, n = 16 on 8 splits: relative error 2.2e-7 ->
-// 1.3e-7, 18.1 -> 18.4 us; m = k = 32768, n = 16: 8.7e-7 -> 3.1e-7, 633 -> 626 us).
+// The tile's chains of fmas cut in eight (at least two stages long each, from eight stages on), their sums totalled apart, for
+// the FP32 widths up to 16: with few splits their chains are long for their k (m = k = 2048, n = 16 on 8 splits: relative
+// error 2.2e-7 -> 1.3e-7, 18.1 -> 18.4 us; m = k = 32768, n = 16: 8.7e-7 -> 3.1e-7, 633 -> 626 us).
 template <typename T, int NP>
 struct TallTotal {
     static constexpr bool ON = sizeof(T) == 4 && NP <= 16;
@@ -305,7 +305,8 @@ struct TallTotal {
     __device__ __forceinline__ explicit TallTotal(int iters) {
         if constexpr (ON) {
             tot.zero();
-            left = seg = iters > 16 ? iters / 8 : 2;
+            seg = iters > 16 ? iters / 8 : 2;
+            left = iters < 8 ? 0 : seg;  // 0: never
         }
     }
     __device__ __forceinline__ void stage(typename TallAcc<T, NP>::type &acc) {
@@ -317,7 +318,8 @@ struct TallTotal {
             }
     }
     __device__ __forceinline__ void finish(typename TallAcc<T, NP>::type &acc) {
-        if constexpr (ON) acc.add(tot);
+        if constexpr (ON)
+            if (left > 0) acc.add(tot);
     }
 };
 
