@@ -514,14 +514,15 @@ def time_points(tsmm, torch, pts, tdt, steps, warmup, precision=0, world=1, rank
     return points, elapsed_ms, launches, state
 
 
-def tensor_products(es, n, k):
+def tensor_products(es, m, n, k):
     """Tensor-core products per product of the native precision, 0 where the FP pipes compute it (the dispatch rules of
-    tsmm_internal.h; FP64 regime (i) also asks for m * n * k >= 4e7)."""
+    tsmm_internal.h: tc_pack and kTcMinK, rank_tc, tc64_plan, rank_tc64)."""
     if es == 4:
-        return 6 if n > 16 and (n <= 64 or k > 32) else 0
+        return 6 if (16 < n <= 64 and k >= 16) or (n > 64 and k > 32) else 0
     if n > 64:
         return 36 if k >= 4 else 0
-    return (28 if n > 48 else 35) if n > 1 and k >= 256 else 0
+    padded = next(w for w in (1, 2, 4, 8, 16, 24, 32, 48, 64) if w >= n)
+    return (28 if n > 48 else 35) if n > 1 and 256 <= k <= 1 << 20 and m * padded * k >= 40_000_000 else 0
 
 
 def bf16_peak():
@@ -547,7 +548,7 @@ def rate_points(points, es, hbm_peak, fp_peak_tf, native=True):
         gb = alg_bytes(rows, n, k, beta, es) / 1e9
         gbs = gb / (ms * 1e-3)
         tf = flops(rows, n, k) / (ms * 1e-3) / 1e12
-        products = tensor_products(es, n, k) if native else 0
+        products = tensor_products(es, rows, n, k) if native else 0
         fp_peak_tf = tensor_tf / products if products else fp_pipe_tf
         bound = "hbm" if gb / hbm_peak >= flops(rows, n, k) / (fp_peak_tf * 1e12) else "alu"
         frac = (gbs / hbm_peak) if bound == "hbm" else (tf / fp_peak_tf)
@@ -612,7 +613,8 @@ def run_ours(args):
     dom = rated[dom_i]
     m, n, k, beta = dom["m"], dom["n"], dom["k"], dom["beta"]
     kernel_key = f"{args.workload}_{args.dtype}_n{n}_k{k}"
-    products = tensor_products(es, n, k) if prec == tsmm.PREC_NATIVE else 0
+    lo, hi = points[dom_i]["rows"]
+    products = tensor_products(es, hi - lo, n, k) if prec == tsmm.PREC_NATIVE else 0
     if products:
         fp_peak_tf = bf16_peak() / products
         fp_src = f"measured dense BF16 peak (MEASURED_PEAKS.json bf16_tflops) / {products} products"
