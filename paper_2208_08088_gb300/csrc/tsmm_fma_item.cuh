@@ -94,7 +94,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
     };
     // Chains of SEG (SEGN) stages, their sums added in `tot`: one chain over a whole item would be several times as long as
     // the fma kernels', whose blocks split k among warps and more splits (FP64, n = 64, k = 2048, uneven columns: error
-    // 5.5e-16, theirs 3.7e-16, so @S@).  The totals sit in shared memory because registers for them spill (FP32,
+    // 5.5e-16, theirs 3.7e-16, so 2.5e-16).  The totals sit in shared memory because registers for them spill (FP32,
     // n = 64: 5 times the time).
     tot += tid;
     // up to 8 columns of FP64 (np <= 8 = HW): the halves share the columns and split each stage's rows, and 16 sums a

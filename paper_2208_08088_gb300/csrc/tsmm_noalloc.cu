@@ -150,7 +150,9 @@ extern "C" tsmm_status tsmm_execute_noalloc(tsmm_dtype dtype, int64_t m, int64_t
     a.slabs = slabs;
     a.arows = 0;
     a.np = np;
-    a.Bt = nullptr;  // the fma kernels (n > 16: their own slab height; the pieces of B would not fit the scratch rule)
+    // The fma kernels at every width.  What this call accepts is bounded by the panel in the scratch; with the pieces or
+    // digits of B beside it n = 64 would fit up to k = 52000 (F32) and 14000 (F64) only.
+    a.Bt = nullptr;
     a.bmin = nullptr;
 
     CUtensorMap tmap;
