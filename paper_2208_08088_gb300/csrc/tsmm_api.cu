@@ -141,6 +141,10 @@ SplitCosts split_costs(tsmm_dtype dt, int np, bool tc, int64_t n) {
 // stages count at one price: there a block's start and the sum over the partials no longer matter, and HBM's rate needs
 // every SM's full count of blocks (m = k = 32768, n = 16: S = 7 takes 611 us and S = 2 667; n = 64 on the tensor cores:
 // 805 and, at S = 1, 852; but m = 30000, n = 48, k = 3000: S = 5 78 us and S = 1 65).
+// Where that switch lies: n = 16 below 64 MB 22.3 us by block costs and 25.9 by waves (48 MB), 24.5 / 26.7 (67), above it 47.4 /
+// 35.7 (134), 81.0 / 55.4 (268).  On the tensor cores the two differ in 29 % of shapes above 1 GB; of 25 such, block costs
+// were faster in 23, by 1 to 3 % in most and 15 to 19 % where k is short (m = 167068, n = 50, k = 2380: S = 1 262 us, S = 2
+// 310), and 9 % slower in one.  The switch stays for the chains of chunk sums, which more splits keep short.
 int choose_splits(const SplitCosts &k, int64_t slabs, int64_t kstages, int num_sms, int64_t max_splits) {
     const int64_t resident = (int64_t)k.resident * num_sms;
     const double bw = 7.0e6;  // bytes per us
