@@ -312,8 +312,8 @@ def run_reference(args):
 
 # --------------------------------------------------------------------- our arm
 KERNEL_SOURCES = {  # the files that define each kernel family's device code
-    "tall": ["tsmm_tall.cuh", "tsmm_tall_tc.cuh", "tsmm_tall_tc64.cuh", "tsmm_digits64.cuh", "tsmm_finish.cuh", "tsmm_tc.cuh",
-             "tsmm_device.cuh"],
+    "tall": ["tsmm_tall.cuh", "tsmm_tall_tc.cuh", "tsmm_tall_tc64.cuh", "tsmm_fma_item.cuh", "tsmm_digits64.cuh", "tsmm_finish.cuh",
+             "tsmm_tc.cuh", "tsmm_device.cuh"],
     "rankk": ["tsmm_rankk.cu", "tsmm_rankk_tc.cu", "tsmm_rankk_tc64.cu", "tsmm_digits64.cuh", "tsmm_tc.cuh",
               "tsmm_device.cuh"],
 }
