@@ -102,7 +102,7 @@ __device__ __forceinline__ void fma_item(const TallArgs &a, int64_t row, int64_t
     const int half = tid / 128;
     auto narrow = [&](auto np_tag) {
         constexpr int NPW = decltype(np_tag)::value, SETS = 16 / NPW < CH / 2 ? 16 / NPW : CH / 2;
-        constexpr int SEGN = 8;
+        constexpr int SEGN = 4 * SETS;  // chains of 32 entries
         FmaAcc<T, NPW> acc[SETS];
 #pragma unroll
         for (int q = 0; q < SETS; ++q) acc[q].zero();

@@ -58,6 +58,11 @@ inline int tall_bm(tsmm_dtype d, int np) { return tall_block_rows(d == TSMM_F64,
 // tiles fit 136 registers), else 2 (the width 48's 8 x 12 tiles need ~160).
 constexpr int tall_resident_blocks(bool f64, int np) { return (!f64 && (np == 32 || np == 64)) ? 3 : 2; }
 
+// Whether the FP32 kernels up to 16 columns cut their chains of fmas (TallTotal): at width 16, whose registers then spill, where A
+// has less than the 64 MB from which the split-K planner fills whole waves as it always did (m = 33868, n = 12, k = 1162: 36.9
+// us without, 38.9 with); below it the planner's splits are fewer than they were, their chains longer.
+__host__ __device__ constexpr bool tall_cut(int np, int64_t m, int64_t k) { return np < 16 || (double)m * (double)k * 4.0 < 64.0e6; }
+
 // FP32 regime (i) with n > 16 runs on the tensor cores (tsmm_tall_tc.cuh): slabs of kTcRows rows, k in chunks of
 // kTcKB, MMA width n rounded up to 16.  The line lies at 16 because up to there the fma kernel streams A at the copy
 // rate (n = 16: 0.64 ms at m = k = 32768), above it does not (n = 20: 0.78 ms against 0.68); m and k need no line

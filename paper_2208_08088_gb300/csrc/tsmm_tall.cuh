@@ -295,18 +295,18 @@ struct TallAcc<float, NP> {
 };
 
 // The tile's chains of fmas cut in eight (at least two stages long each, from eight stages on), their sums totalled apart, for
-// the FP32 widths up to 16: with few splits their chains are long for their k (m = k = 2048, n = 16 on 8 splits: relative
-// error 2.2e-7 -> 1.3e-7, 18.1 -> 18.4 us; m = k = 32768, n = 16: 8.7e-7 -> 3.1e-7, 633 -> 626 us).
-template <typename T, int NP>
+// the FP32 widths up to 16 (tall_cut): with few splits their chains are long for their k (m = k = 2048, n = 16 on 8 splits:
+// relative error 2.2e-7 -> 1.3e-7, 18.1 -> 18.4 us; m = k = 32768, n = 1: 8.7e-7 -> 3.1e-7 in the same time).
+template <typename T, int NP, bool CUT>
 struct TallTotal {
-    static constexpr bool ON = sizeof(T) == 4 && NP <= 16;
+    static constexpr bool ON = CUT && sizeof(T) == 4 && NP <= 16;
     typename TallAcc<T, NP>::type tot;
     int seg, left;
-    __device__ __forceinline__ explicit TallTotal(int iters) {
+    __device__ __forceinline__ TallTotal(int iters, const TallArgs &a) {
         if constexpr (ON) {
             tot.zero();
             seg = iters > 16 ? iters / 8 : 2;
-            left = iters < 8 ? 0 : seg;  // 0: never
+            left = iters < 8 || !tall_cut(NP, a.m, a.k) ? 0 : seg;  // 0: never
         }
     }
     __device__ __forceinline__ void stage(typename TallAcc<T, NP>::type &acc) {
@@ -322,11 +322,16 @@ struct TallTotal {
             if (left > 0) acc.add(tot);
     }
 };
+// Single problems that never cut have a kernel without the totals (the grouped kernel asks per problem).
+template <typename T, int NP>
+bool tall_uncut(const TallArgs &a) {
+    return sizeof(T) == 4 && NP == 16 && !tall_cut(NP, a.m, a.k);
+}
 
 // One block's work item (m-slab `slab`, k range `split`) with A described by
 // the tensor map *tmA (a kernel parameter); the body of the single-problem
 // kernel and of the grouped kernel.
-template <typename T, int NP>
+template <typename T, int NP, bool CUT = true>
 __device__ __forceinline__ void tall_tma_block(const CUtensorMap *tmA, const TallArgs &a, int64_t slab,
                                                int split) {
     using Cfg = TallCfg<T, NP>;
@@ -390,7 +395,7 @@ __device__ __forceinline__ void tall_tma_block(const CUtensorMap *tmA, const Tal
 
     typename TallAcc<T, NP>::type acc;
     acc.zero();
-    TallTotal<T, NP> total(iters);
+    TallTotal<T, NP, CUT> total(iters, a);
 
     bool ok = true;
     for (int it = 0; it < iters; ++it) {
@@ -434,10 +439,10 @@ __device__ __forceinline__ void tall_tma_block(const CUtensorMap *tmA, const Tal
     tall_finish<T, NP>(red, a, slab, split, threadIdx.x, flag);
 }
 
-template <typename T, int NP>
+template <typename T, int NP, bool CUT = true>
 __global__ void __launch_bounds__(TallCfg<T, NP>::THREADS, TallCfg<T, NP>::RESIDENT)
     tall_tma_kernel(const __grid_constant__ CUtensorMap tmA, const TallArgs a) {
-    tall_tma_block<T, NP>(&tmA, a, blockIdx.x, (int)blockIdx.y);
+    tall_tma_block<T, NP, CUT>(&tmA, a, blockIdx.x, (int)blockIdx.y);
 }
 
 // Same decomposition without a tensor map, for an A that one cannot describe
@@ -511,7 +516,7 @@ __device__ __forceinline__ Vec<float, Cfg::R> load_rows_at(const float *slot, in
 // column c of a stage sits (c * LV) mod 4 elements into its slot, known at
 // compile time, and its rows are read with load_rows_at.  LV = -1: any A, the
 // offsets computed at run time and the rows read element by element.
-template <typename T, int NP, int LV = -1>
+template <typename T, int NP, int LV = -1, bool CUT = true>
 __device__ __forceinline__ void tall_async_block(const TallArgs &a, int64_t slab, int split) {
     using Cfg = TallCfg<T, NP>;
     using AC = AsyncCfg<T, NP>;
@@ -595,7 +600,7 @@ __device__ __forceinline__ void tall_async_block(const TallArgs &a, int64_t slab
     const int cloc = g * Cfg::CN;
     typename TallAcc<T, NP>::type acc;
     acc.zero();
-    TallTotal<T, NP> total(iters);
+    TallTotal<T, NP, CUT> total(iters, a);
     // every stage starts at a multiple of BKS (k splits are whole stages), so a
     // column's offset within 16 bytes depends only on its index mod V
     int doff[V];
@@ -650,35 +655,39 @@ __device__ __forceinline__ void tall_async_block(const TallArgs &a, int64_t slab
     tall_finish<T, NP>(red, a, slab, split, threadIdx.x, flag);
 }
 
-template <typename T, int NP, int LV>
+template <typename T, int NP, int LV, bool CUT = true>
 __global__ void __launch_bounds__(TallCfg<T, NP>::THREADS, TallCfg<T, NP>::RESIDENT)
     tall_async_kernel(const TallArgs a) {
-    tall_async_block<T, NP, LV>(a, blockIdx.x, (int)blockIdx.y);
+    tall_async_block<T, NP, LV, CUT>(a, blockIdx.x, (int)blockIdx.y);
 }
 
-template <typename T, int NP>
+template <typename T, int NP, bool CUT = true>
 cudaError_t launch_tall_tma_t(const CUtensorMap *tmap, const TallArgs &a, cudaStream_t s) {
     using Cfg = TallCfg<T, NP>;
+    if constexpr (CUT && sizeof(T) == 4 && NP == 16)
+        if (tall_uncut<T, NP>(a)) return launch_tall_tma_t<T, NP, false>(tmap, a, s);
     {
         const cudaError_t e =
-            ensure_smem_limit(reinterpret_cast<const void *>(tall_tma_kernel<T, NP>), Cfg::SMEM);
+            ensure_smem_limit(reinterpret_cast<const void *>(tall_tma_kernel<T, NP, CUT>), Cfg::SMEM);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)a.slabs, (unsigned)a.splits);
-    tall_tma_kernel<T, NP><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(*tmap, a);
+    tall_tma_kernel<T, NP, CUT><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(*tmap, a);
     return cudaGetLastError();
 }
 
-template <typename T, int NP, int LV>
+template <typename T, int NP, int LV, bool CUT = true>
 cudaError_t launch_tall_async_lv(const TallArgs &a, cudaStream_t s) {
     const int smem = AsyncCfg<T, NP>::SMEM;
+    if constexpr (CUT && sizeof(T) == 4 && NP == 16)
+        if (tall_uncut<T, NP>(a)) return launch_tall_async_lv<T, NP, LV, false>(a, s);
     {
         const cudaError_t e =
-            ensure_smem_limit(reinterpret_cast<const void *>(tall_async_kernel<T, NP, LV>), smem);
+            ensure_smem_limit(reinterpret_cast<const void *>(tall_async_kernel<T, NP, LV, CUT>), smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)a.slabs, (unsigned)a.splits);
-    tall_async_kernel<T, NP, LV><<<grid, TallCfg<T, NP>::THREADS, smem, s>>>(a);
+    tall_async_kernel<T, NP, LV, CUT><<<grid, TallCfg<T, NP>::THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
